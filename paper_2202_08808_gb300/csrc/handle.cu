@@ -427,9 +427,8 @@ struct dspg_handle {
     // buffer allocates for the call instead of holding that memory
     struct ReadWs {
         DBuf<int32_t> rows, lens, c, r;
-        DBuf<int64_t> rp, scan, listed, st, so, chunk_cnt, chunk_ex, chunk_tmp, long_l, huge_l;
+        DBuf<int64_t> rp, scan, st, so, chunk_cnt, chunk_ex, chunk_tmp, long_l, huge_l;
         DBuf<ReadOut> res;
-        DBuf<unsigned> n_listed;
         DBuf<char> v;
         DBuf<uint64_t> k0, k1;
         DBuf<uint32_t> i0, i1, counts;
@@ -1391,37 +1390,38 @@ void sort_listed_host(dspg_handle *h, const DevMat &M, const int64_t *rp, const 
 
 void fill_rows_out(dspg_handle *h, DevMat &M, const MatView &V, int vs, const int32_t *rows, int64_t n, int64_t *rp,
                    int64_t nnz, int64_t *rowptr, int32_t *col, void *val, int on_device, cudaStream_t s) {
-    // rows too long to sort in shared memory are listed, then sorted together
+    // rows of more than 64 entries are listed; of those, in a very wide C,
+    // the ones too long to sort in shared memory, which are then sorted together
     const int64_t list_cap = nnz / 16385 + 1;
-    DBuf<int64_t> listed_l;
-    h->rd.n_listed.reserve(1);
-    unsigned *n_listed = h->rd.n_listed.p;
-    int64_t *listed = read_scratch(h->rd.listed, listed_l, list_cap);
-    CK(cudaMemsetAsync(n_listed, 0, sizeof(unsigned), s));
-    auto sort_out = [&](int32_t *oc, void *ov) {
-        sort_rows(rp, n, oc, ov, vs, n_listed, listed, list_cap, s, h->num_sms);
-        unsigned nl = 0;
-        CK(cudaMemcpyAsync(&nl, n_listed, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+    DBuf<int64_t> long_l, huge_l;
+    int64_t *longs = read_scratch(h->rd.long_l, long_l, std::min<int64_t>(n, nnz / 65) + 1);
+    int64_t *huge = read_scratch(h->rd.huge_l, huge_l, list_cap);
+    h->rd.res.reserve(1);
+    CK(cudaMemsetAsync(h->rd.res.p, 0, sizeof(ReadOut), s));
+    auto rows_out = [&](int32_t *oc, void *ov) {
+        read_rows_out(rows, n, nullptr, V, vs, rp, nullptr, nnz, oc, ov, nullptr, nullptr, longs, huge, h->rd.res.p, s,
+                      h->num_sms);
+        ReadOut ro{};
+        CK(cudaMemcpyAsync(&ro, h->rd.res.p, sizeof(ReadOut), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
+        const unsigned nl = ro.n_huge;
         if (nl == 0) return;
         if ((int64_t)nl > list_cap) throw Err(DSPG_ERR_CUDA, "more long rows than the read can hold");
         std::vector<int64_t> lh(nl), rph(n + 1);
-        CK(cudaMemcpyAsync(lh.data(), listed, sizeof(int64_t) * nl, cudaMemcpyDeviceToHost, s));
+        CK(cudaMemcpyAsync(lh.data(), huge, sizeof(int64_t) * nl, cudaMemcpyDeviceToHost, s));
         CK(cudaMemcpyAsync(rph.data(), rp, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
         sort_listed_host(h, M, rp, lh, rph.data(), oc, ov, vs, s);
     };
     if (on_device) {
         CK(cudaMemcpyAsync(rowptr, rp, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToDevice, s));
-        gather_rows_out(rows, n, V, rp, col, val, vs, s, h->num_sms);
-        sort_out(col, val);
+        rows_out(col, val);
     } else {
         DBuf<int32_t> c_l;
         DBuf<char> v_l;
         int32_t *c = read_scratch(h->rd.c, c_l, nnz);
         char *v = read_scratch(h->rd.v, v_l, nnz * std::max(vs, 1));
-        gather_rows_out(rows, n, V, rp, c, v, vs, s, h->num_sms);
-        sort_out(c, vs ? (void *)v : nullptr);
+        rows_out(c, vs ? (void *)v : nullptr);
         CK(cudaMemcpyAsync(rowptr, rp, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToHost, s));
         if (nnz > 0) {
             if (col) CK(cudaMemcpyAsync(col, c, sizeof(int32_t) * nnz, cudaMemcpyDeviceToHost, s));
@@ -2542,10 +2542,11 @@ dspg_status dspg_fault_inject(const char *spec) {
     return DSPG_OK;
 }
 
-// The end of a direct read whose rows over 16384 entries were out of order
-// (ro.n_huge of them, listed in the read's scratch): each is sorted in the
-// scratch on the device and copied into the caller's col and val (rp: the
-// device row pointers, rowptr: the same on the host).
+// The end of a direct read of a very wide C whose rows over 16384 entries
+// were out of order (ro.n_huge of them, listed, as they are in the read's
+// scratch): each is sorted in the scratch on the device and copied into the
+// caller's col and val (rp: the device row pointers, rowptr: the same on
+// the host).
 static void read_huge_rows(dspg_handle *h, const ReadOut &ro, const int64_t *rp, const int64_t *rowptr,
                            int32_t *col, void *val, cudaStream_t s) {
     dspg_handle::ReadWs &w = h->rd;
@@ -2617,8 +2618,8 @@ dspg_status dspg_read_affected_C(dspg_handle *h, int64_t rows_cap, int64_t nnz_c
             w.huge_l.reserve(std::max<int64_t>(n, 1));
             w.c.reserve(std::max<int64_t>(nnz_cap, 1));
             w.v.reserve(std::max<int64_t>(nnz_cap, 1) * std::max(h->vsize, 1));
-            read_rows_direct(w.r.p, n, nullptr, h->C.view(), h->vsize, rp, w.chunk_ex.p + nch, nnz_cap, dcol, dval,
-                             w.c.p, (void *)w.v.p, w.long_l.p, w.huge_l.p, w.res.p, s, h->num_sms);
+            read_rows_out(w.r.p, n, nullptr, h->C.view(), h->vsize, rp, w.chunk_ex.p + nch, nnz_cap, w.c.p,
+                          (void *)w.v.p, dcol, dval, w.long_l.p, w.huge_l.p, w.res.p, s, h->num_sms);
             ReadOut ro{};
             CK(cudaMemcpyAsync(&ro, w.res.p, sizeof(ReadOut), cudaMemcpyDeviceToHost, s));
             if (n > 0 && !drows) CK(cudaMemcpyAsync(rows, w.r.p, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, s));
@@ -2721,8 +2722,8 @@ dspg_status dspg_apply_read_affected(dspg_handle *h, const dspg_updates *dA, con
                 read_order_rowptr(h->wc.R.p, h->wc.rchunk.p, nch, rc, n_dev, cap, &h->ctl->status, h->C.len.p, w.r.p,
                                   w.lens.p, w.chunk_cnt.p, w.chunk_ex.p + nch, w.rp.p, drows, drp, w.res.p, s,
                                   h->num_sms);
-                read_rows_direct(w.r.p, rc, n_dev, h->C.view(), h->vsize, w.rp.p, w.chunk_ex.p + nch, nnz_cap, dcol,
-                                 dval, w.c.p, (void *)w.v.p, w.long_l.p, w.huge_l.p, w.res.p, s, h->num_sms);
+                read_rows_out(w.r.p, rc, n_dev, h->C.view(), h->vsize, w.rp.p, w.chunk_ex.p + nch, nnz_cap, w.c.p,
+                              (void *)w.v.p, dcol, dval, w.long_l.p, w.huge_l.p, w.res.p, s, h->num_sms);
                 CK(cudaMemcpyAsync(&ro, w.res.p, sizeof(ReadOut), cudaMemcpyDeviceToHost, s));
                 CK(cudaStreamSynchronize(s));
                 // a batch that needs a second pass changes C after the read

@@ -280,12 +280,6 @@ void copy_rows(const int32_t *rows, int64_t n, const int64_t *src_off, const int
                cudaStream_t s, int num_sms);
 void gather_rows_out(const int32_t *rows, int64_t n, const MatView &M, const int64_t *out_rowptr, int32_t *out_col,
                      void *out_val, int vsize, cudaStream_t s, int num_sms);
-// Sort each row of a gathered CSR (rowptr over n rows) by column, in place;
-// rows longer than 16384 entries that are out of order are counted in
-// *n_listed and their indices written to listed[0, list_cap) instead, for
-// sort_listed_rows.
-void sort_rows(const int64_t *rowptr, int64_t n, int32_t *col, void *val, int vsize, unsigned *n_listed,
-               int64_t *listed, int64_t list_cap, cudaStream_t s, int num_sms);
 struct SortScratch {  // for `total` entries: keys, indices (two each), radix counts, scans, gather space
     uint64_t *k0, *k1;
     uint32_t *i0, *i1, *counts;
@@ -298,27 +292,30 @@ struct SortScratch {  // for `total` entries: keys, indices (two each), radix co
 void sort_listed_rows(const int64_t *rowptr, const int64_t *listed, const int64_t *pre, int nl, int64_t total,
                       int cb, int32_t *col, void *val, int vsize, const SortScratch &w, cudaStream_t s, int num_sms);
 void lens_of_rows(const int32_t *rows, int64_t n, const int32_t *len, int32_t *out, cudaStream_t s);
-// A read of rows of C straight into page-locked host buffers (layout.cu):
-// what it found, for the one host synchronisation after it.
+// What a read of rows found (layout.cu), for the host synchronisation after it.
 struct ReadOut {
     long long nnz;   // entries of the rows (rp[n])
     unsigned n_long; // rows of more than 64 entries (listed)
-    unsigned n_huge; // of those, rows over 16384 entries that are out of order (left in the scratch)
+    unsigned n_huge; // of those, in a very wide C, rows over 16384 entries that are out of order (left in dst)
     unsigned flags;  // READ_TOO_SMALL, READ_UNORDERED: nothing was written
-    unsigned pad;
+    unsigned next;   // ticket of the next listed row
     long long nr;    // the rows of R (n, as read on the device)
 };
 enum : unsigned { READ_TOO_SMALL = 1u, READ_UNORDERED = 2u };
-// rows[0..n) (ascending, R from its collection when r_total is given: its
-// chunk total must equal n), their row pointers rp (device, rp[n] = entries)
-// -> out_col/out_val (device addresses of page-locked host memory, at least
-// nnz_cap entries; out_val may be null).  Scratch: nnz_cap entries; lists:
-// n entries each; res zeroed by the caller.
+// rows[0..n) of M (every row when rows is null; when r_total is given, R
+// from its collection, whose chunk total must equal n) in column order, at
+// the row pointers rp (device, rp[n] = entries): into dst_col/dst_val
+// (device, nnz_cap entries), or into out_col/out_val when given (device
+// addresses of page-locked host memory, at least nnz_cap entries), with dst
+// as the scratch of the longer rows.  The values' array may be null: then
+// columns only.  Lists: one entry per row of more than 64 entries
+// (long_list), and in a C of more than 2^22 columns per row of more than
+// 16384 (huge_list); res zeroed by the caller.
 // n_dev (or null): n read on the device, n then bounding it (grid sizes).
-void read_rows_direct(const int32_t *rows, int64_t n, const long long *n_dev, const MatView &M, int vsize,
-                      const int64_t *rp, const int64_t *r_total, int64_t nnz_cap, int32_t *out_col, void *out_val,
-                      int32_t *scr_col, void *scr_val, int64_t *long_list, int64_t *huge_list, ReadOut *res,
-                      cudaStream_t s, int num_sms);
+void read_rows_out(const int32_t *rows, int64_t n, const long long *n_dev, const MatView &M, int vsize,
+                   const int64_t *rp, const int64_t *r_total, int64_t nnz_cap, int32_t *dst_col, void *dst_val,
+                   int32_t *out_col, void *out_val, int64_t *long_list, int64_t *huge_list, ReadOut *res,
+                   cudaStream_t s, int num_sms);
 // R (n rows, as collected: ascending within each 8192-row chunk, chunk c's
 // rows at chunk[2c] with chunk[2c+1] of them) into out in row order; cnt and
 // ex (nch + 1) and tmp (scan_tmp_entries(nch) + 1) are scratch, and ex[nch]

@@ -333,45 +333,289 @@ void gather_rows_out(const int32_t *rows, int64_t n, const MatView &M, const int
     else launch_k(k_gather_out<int32_t>, g, 256, 0, s, rows, n, M, out_rowptr, out_col, (int32_t *)out_val);
 }
 
-// ------------------------------------------------------- row sorting
+// ------------------------------------------------- rows out, in column order
 
 // C's rows are stored in any column order (the hash bins write long rows in
-// table order); every read returns canonical rows, so the gathered rows are
-// sorted by column here.  Rows already in order are left as they are.
+// table order); every read returns canonical rows.  Two launches take the
+// rows straight from the arena to their places in the result, which is
+// device memory or, through the C2C link, the caller's page-locked arrays:
+// k_read_short the rows of up to SORT_SHORT entries, which it also counts
+// and lists the longer ones of, and k_order_long (or k_sort_long where C is
+// very wide) those.
 constexpr int SORT_SHORT = 64;     // rows up to this length: a warp each
-constexpr int SORT_MAX = 16384;    // longer rows are listed and sorted together (sort_listed_rows)
+constexpr int SORT_MAX = 16384;    // very wide C: longer rows are listed and sorted together (sort_listed_rows)
+constexpr int RS_NT = 256;         // threads of a k_read_short block
+constexpr int RS_ROWS = 32;        // rows of its tile
+constexpr int RS_PW = RS_ROWS / (RS_NT / 32);  // rows of a warp
+
+// A tile of RS_ROWS consecutive rows per block and round: each warp loads
+// its four rows together, ranks the columns of those out of order by
+// shuffles, and puts the entries at their places in shared memory; the
+// block then stores the tile's stretch of the result, whole 128-byte lines
+// at a time.  What bounds it is the far side of the stores: into host
+// memory rows stored one by one (each starting and ending inside a line)
+// reached 144 GB/s on the rows of a 10^4-update stencil batch (17.5 MB: 122
+// us) against the link's 190; now 95 us.  Into device memory it is one pass
+// instead of a gather and an in-place sort (the 51.7 million entries of the
+// 128^3 stencil's square: 0.39 instead of 1.41 ms).  A tile with a longer row
+// stores its short rows directly.  Nothing is written when R is not the
+// ordered list of its collection (r_total != n) or the entries do not fit
+// nnz_cap; the flags say which.
+template <typename T>
+__global__ void __launch_bounds__(RS_NT)
+k_read_short(const int32_t *rows, int64_t n_arg, const long long *n_dev, MatView M, const int64_t *rp,
+             const int64_t *r_total, int64_t nnz_cap, int32_t *out_col, T *out_val, int64_t *long_list, ReadOut *res) {
+    pdl_begin();
+    __shared__ T s_val[RS_ROWS * SORT_SHORT];
+    __shared__ int32_t s_col[RS_ROWS * SORT_SHORT];
+    const int64_t n = n_dev ? (int64_t)*n_dev : n_arg;
+    // rp[n] exists only when R was placed (r_total == n)
+    const bool unordered = r_total && *r_total != n;
+    const int64_t nnz = unordered ? 0 : rp[n];
+    const unsigned bad = (unordered ? READ_UNORDERED : 0u) | (nnz > nnz_cap ? READ_TOO_SMALL : 0u);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        res->nnz = nnz;
+        if (bad) atomicOr(&res->flags, bad);
+    }
+    if (bad) return;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const T *mv = (const T *)M.val;
+    for (int64_t x0 = (int64_t)blockIdx.x * RS_ROWS; x0 < n; x0 += (int64_t)gridDim.x * RS_ROWS) {
+        const int64_t x1 = x0 + RS_ROWS < n ? x0 + RS_ROWS : n;
+        const int64_t base = rp[x0], end = rp[x1];
+        // lanes 0..RS_PW - 1 hold the warp's rows
+        int64_t h_so = 0, h_d = 0;
+        int64_t h_len = 0;
+        const int64_t hx = x0 + w * RS_PW + lane;
+        if (lane < RS_PW && hx < x1) {
+            h_d = rp[hx];
+            h_len = rp[hx + 1] - h_d;
+            h_so = M.off[rows ? (int64_t)rows[hx] : hx];
+        }
+        const bool lng = h_len > SORT_SHORT;
+        const unsigned lm = __ballot_sync(0xffffffffu, lng);
+        if (lm) {  // the long rows of this warp: one atomic
+            unsigned at = 0;
+            if (lane == 0) at = atomicAdd(&res->n_long, (unsigned)__popc(lm));
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (lng) long_list[at + __popc(lm & lanemask_lt())] = hx;
+        }
+        const bool staged = !__syncthreads_or(lng);  // then the tile has at most RS_ROWS * SORT_SHORT entries
+        const int len_l = lng ? 0 : (int)h_len;
+        int len[RS_PW];
+        int32_t k0[RS_PW], k1[RS_PW];
+        T v0[RS_PW], v1[RS_PW];
+#pragma unroll
+        for (int j = 0; j < RS_PW; j++) {  // every load of the warp's rows before any use
+            const int L = __shfl_sync(0xffffffffu, len_l, j);
+            const int64_t so = __shfl_sync(0xffffffffu, h_so, j);
+            len[j] = L;
+            k0[j] = lane < L ? M.col[so + lane] : INT32_MAX;
+            k1[j] = lane + 32 < L ? M.col[so + lane + 32] : INT32_MAX;
+            v0[j] = out_val && lane < L ? mv[so + lane] : T(0);
+            v1[j] = out_val && lane + 32 < L ? mv[so + lane + 32] : T(0);
+        }
+#pragma unroll
+        for (int j = 0; j < RS_PW; j++) {
+            const int L = len[j];
+            const int64_t d = __shfl_sync(0xffffffffu, h_d, j);
+            // entry e + 1 after entry e: the next lane's, across the halves at lane 31
+            const int32_t up0 = __shfl_down_sync(0xffffffffu, k0[j], 1);
+            const int32_t lo1 = __shfl_sync(0xffffffffu, k1[j], 0);
+            const int32_t up1 = __shfl_down_sync(0xffffffffu, k1[j], 1);
+            const int32_t n0 = lane == 31 ? lo1 : up0;
+            const bool out_of_order = (lane + 1 < L && k0[j] > n0) || (lane + 33 < L && k1[j] > up1);
+            int r0 = lane, r1 = lane + 32;
+            if (__any_sync(0xffffffffu, out_of_order)) {  // rank among the row's (distinct) columns
+                r0 = 0;
+                r1 = 0;
+                for (int q = 0; q < 32; q++) {
+                    const int32_t a = __shfl_sync(0xffffffffu, k0[j], q), b = __shfl_sync(0xffffffffu, k1[j], q);
+                    r0 += (a < k0[j]) + (b < k0[j]);
+                    r1 += (a < k1[j]) + (b < k1[j]);
+                }
+            }
+            if (staged) {
+                const int o = (int)(d - base);
+                if (lane < L) {
+                    s_col[o + r0] = k0[j];
+                    s_val[o + r0] = v0[j];
+                }
+                if (lane + 32 < L) {
+                    s_col[o + r1] = k1[j];
+                    s_val[o + r1] = v1[j];
+                }
+            } else {
+                if (lane < L) {
+                    out_col[d + r0] = k0[j];
+                    if (out_val) out_val[d + r0] = v0[j];
+                }
+                if (lane + 32 < L) {
+                    out_col[d + r1] = k1[j];
+                    if (out_val) out_val[d + r1] = v1[j];
+                }
+            }
+        }
+        if (staged) {
+            __syncthreads();
+            // from the 32-entry boundary at or below base, so that a warp's stores fill lines
+            const int cnt = (int)(end - base);
+            for (int i = tid - (int)(base & 31); i < cnt; i += RS_NT)
+                if (i >= 0) {
+                    out_col[base + i] = s_col[i];
+                    if (out_val) out_val[base + i] = s_val[i];
+                }
+        }
+        __syncthreads();
+    }
+}
+
+// The listed rows of more than SORT_SHORT entries, a block each (taken by a
+// ticket, as their lengths differ by orders of magnitude).  The columns of a
+// row are distinct, so the place of an entry in column order is the number
+// of the row's columns below its own: the columns are marked in a bitmap in
+// shared memory, the marks counted (per 1024 columns by the marking itself,
+// inside those by a warp each, only where there are any), and each entry
+// looks up the marks below its bit and goes straight to its place.  Work per
+// row: its entries three times from L1/L2 and two shared-memory atomics per
+// entry, against the log^2 passes of a sorting network over the next power
+// of two (300-edge batches of R-MAT 18, 27 million entries in rows of 2,000
+// on average into host memory: 4.2 ms with the network in 196 KB of shared
+// memory, one block per SM; 1.55 ms now, the link's rate.  A warp's register
+// network for rows of up to 512 entries measured the same in every case).  Columns are taken in windows of W, from the row's first to its
+// last, and a window keeps 4 blocks of 512 threads on an SM (50 KB at
+// W = 2^18, OL_W).  A row already in order (the dense kernels' rows) is
+// copied.  With host arrays (out_col) the row is put together in device
+// memory (dst_col, dst_val: it stays in L2) and stored to the host in order.
+constexpr int OL_NT = 512;
+constexpr int OL_W = 1 << 18;          // columns of a window
+// C wider than this: k_sort_long.  A row then takes up to 16 windows of about
+// 2 us each, what the network takes for rows of 512 to 1024 entries.
+constexpr int64_t OL_MAX_COLS = (int64_t)1 << 22;
+
+static size_t order_long_smem(int W) { return (size_t)W / 32 * 6 + (size_t)W / 1024 * 8; }
 
 template <typename T>
-__global__ void k_sort_short_rows(const int64_t *rowptr, int64_t n, int32_t *col, T *val) {
+__global__ void __launch_bounds__(OL_NT)
+k_order_long(const int32_t *rows, MatView M, const int64_t *rp, const int64_t *long_list, int32_t *dst_col, T *dst_val,
+             int32_t *out_col, T *out_val, bool has_val, ReadOut *res, int W) {
     pdl_begin();
-    const int lane = threadIdx.x & 31;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < n; x += nwarps) {
-        const int64_t lo = rowptr[x];
-        const int len = (int)(rowptr[x + 1] - lo);
-        if (len < 2 || len > SORT_SHORT) continue;
-        const int32_t k0 = lane < len ? col[lo + lane] : INT32_MAX;
-        const int32_t k1 = lane + 32 < len ? col[lo + lane + 32] : INT32_MAX;
-        T v0 = T(0), v1 = T(0);
-        if (val) {
-            if (lane < len) v0 = val[lo + lane];
-            if (lane + 32 < len) v1 = val[lo + lane + 32];
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint32_t *bm = (uint32_t *)smem;          // W / 32 words: the marked columns of the window
+    uint32_t *cnt = bm + W / 32;              // W / 1024: marks per 1024 columns
+    uint32_t *first = cnt + W / 1024;         // W / 1024: marks before them
+    uint16_t *pre = (uint16_t *)(first + W / 1024);  // W / 32: marks before a word inside its 1024 columns
+    __shared__ unsigned s_t;
+    __shared__ int s_mn, s_mx;
+    __shared__ uint32_t s_w[OL_NT / 32 + 1];
+    if (res->flags) return;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const unsigned nl = res->n_long;
+    const T *mv = (const T *)M.val;
+    for (int q = tid; q < W / 32; q += OL_NT) bm[q] = 0u;
+    for (int q = tid; q < W / 1024; q += OL_NT) cnt[q] = 0u;
+    while (true) {
+        if (tid == 0) {
+            s_t = atomicAdd(&res->next, 1u);
+            s_mn = INT32_MAX;
+            s_mx = -1;
         }
-        // rank of each key among the row's (distinct) columns
-        int r0 = 0, r1 = 0;
-        for (int j = 0; j < 32; j++) {
-            const int32_t a = __shfl_sync(0xffffffffu, k0, j), b = __shfl_sync(0xffffffffu, k1, j);
-            r0 += (a < k0) + (b < k0);
-            r1 += (a < k1) + (b < k1);
+        __syncthreads();
+        const unsigned t = s_t;
+        if (t >= nl) return;
+        const int64_t x = long_list[t];
+        const int64_t lo = rp[x];
+        const int64_t len = rp[x + 1] - lo;
+        const int64_t so = M.off[rows ? (int64_t)rows[x] : x];
+        const int32_t *mc = M.col + so;
+        int unsorted = 0;
+        int mn = INT32_MAX, mx = -1;
+#pragma unroll 4
+        for (int64_t e = tid; e < len; e += OL_NT) {
+            const int32_t c = mc[e];
+            const int32_t nx = e + 1 < len ? mc[e + 1] : INT32_MAX;
+            unsorted |= c > nx;
+            mn = min(mn, c);
+            mx = max(mx, c);
         }
-        __syncwarp();
-        if (lane < len) {
-            col[lo + r0] = k0;
-            if (val) val[lo + r0] = v0;
+        mn = __reduce_min_sync(0xffffffffu, mn);
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        if (lane == 0) {
+            atomicMin(&s_mn, mn);
+            atomicMax(&s_mx, mx);
         }
-        if (lane + 32 < len) {
-            col[lo + r1] = k1;
-            if (val) val[lo + r1] = v1;
+        if (!__syncthreads_or(unsorted)) {
+            int32_t *oc = out_col ? out_col : dst_col;
+            T *ov = out_col ? out_val : dst_val;
+#pragma unroll 4
+            for (int64_t e = tid - (int64_t)(lo & 31); e < len; e += OL_NT)
+                if (e >= 0) {
+                    oc[lo + e] = mc[e];
+                    if (has_val) ov[lo + e] = mv[so + e];
+                }
+            __syncthreads();  // every thread has read s_t, s_mn and s_mx
+            continue;
+        }
+        mn = s_mn;
+        mx = s_mx;
+        uint32_t carry = 0;  // entries of the windows before
+        for (int wb = mn & ~1023; wb <= mx; wb += W) {
+            const int nb = min(W, (mx - wb + 1024) & ~1023) >> 10;  // 1024-column stretches of this window
+#pragma unroll 4
+            for (int64_t e = tid; e < len; e += OL_NT) {
+                const uint32_t c = (uint32_t)(mc[e] - wb);
+                if (c < (uint32_t)W) {
+                    atomicOr(&bm[c >> 5], 1u << (c & 31));
+                    atomicAdd(&cnt[c >> 10], 1u);
+                }
+            }
+            __syncthreads();
+            for (int b = w; b < nb; b += OL_NT / 32)
+                if (cnt[b]) {
+                    const uint32_t p = __popc(bm[b * 32 + lane]);
+                    pre[b * 32 + lane] = (uint16_t)(warp_incl_scan<uint32_t>(p) - p);
+                }
+            // marks before each stretch: nb <= OL_W / 1024 <= OL_NT, one a thread
+            const uint32_t v = tid < nb ? cnt[tid] : 0u;
+            const uint32_t incl = warp_incl_scan<uint32_t>(v);
+            if (lane == 31) s_w[w] = incl;
+            __syncthreads();
+            if (w == 0) {
+                const uint32_t a = lane < OL_NT / 32 ? s_w[lane] : 0u;
+                const uint32_t ai = warp_incl_scan<uint32_t>(a);
+                if (lane < OL_NT / 32) s_w[lane] = ai - a;
+                if (lane == 31) s_w[OL_NT / 32] = ai;
+            }
+            __syncthreads();
+            if (tid < nb) first[tid] = carry + s_w[w] + incl - v;
+            carry += s_w[OL_NT / 32];
+            __syncthreads();
+#pragma unroll 4
+            for (int64_t e = tid; e < len; e += OL_NT) {
+                const int32_t col = mc[e];
+                const uint32_t c = (uint32_t)(col - wb);
+                if (c < (uint32_t)W) {
+                    const int64_t o = lo + first[c >> 10] + pre[c >> 5] + __popc(bm[c >> 5] & ((1u << (c & 31)) - 1u));
+                    dst_col[o] = col;
+                    if (has_val) dst_val[o] = mv[so + e];
+                }
+            }
+            __syncthreads();
+            for (int b = w; b < nb; b += OL_NT / 32)
+                if (cnt[b]) {
+                    bm[b * 32 + lane] = 0u;
+                    __syncwarp();
+                    if (lane == 0) cnt[b] = 0u;
+                }
+            __syncthreads();
+        }
+        if (out_col) {
+#pragma unroll 4
+            for (int64_t e = tid - (int64_t)(lo & 31); e < len; e += OL_NT)
+                if (e >= 0) {
+                    out_col[lo + e] = __ldcg(dst_col + lo + e);
+                    if (has_val) out_val[lo + e] = __ldcg(dst_val + lo + e);
+                }
         }
     }
 }
@@ -402,127 +646,14 @@ __device__ __forceinline__ void block_sort_row(int32_t *sk, T *sv, int N, bool h
     }
 }
 
+// The listed rows of a C wider than OL_MAX_COLS, a block each: put in column
+// order in shared memory (unless in order already); rows over SORT_MAX
+// entries are copied as they are to dst and listed again (huge_list) for
+// sort_listed_rows.
 template <typename T>
-__global__ void __launch_bounds__(512) k_sort_long_rows(const int64_t *rowptr, int64_t n, int32_t *col, T *val,
-                                                        unsigned *n_listed, int64_t *listed, int64_t list_cap) {
-    pdl_begin();
-    extern __shared__ __align__(16) unsigned char smem[];
-    T *sv = (T *)smem;
-    int32_t *sk = (int32_t *)(sv + SORT_MAX);
-    const int tid = threadIdx.x, nt = blockDim.x;
-    for (int64_t x = blockIdx.x; x < n; x += gridDim.x) {
-        const int64_t lo = rowptr[x];
-        const int64_t len = rowptr[x + 1] - lo;
-        if (len <= SORT_SHORT) continue;
-        int unsorted = 0;
-        for (int64_t e = tid; e + 1 < len; e += nt) unsorted |= col[lo + e] > col[lo + e + 1];
-        if (!__syncthreads_or(unsorted)) continue;
-        if (len > SORT_MAX) {  // too long for shared memory: listed for sort_listed_rows
-            if (tid == 0) {
-                const unsigned k = atomicAdd(n_listed, 1u);
-                if (k < list_cap) listed[k] = x;
-            }
-            continue;
-        }
-        int N = 128;
-        while (N < len) N <<= 1;
-        for (int e = tid; e < N; e += nt) {
-            sk[e] = e < len ? col[lo + e] : INT32_MAX;
-            if (val && e < len) sv[e] = val[lo + e];
-        }
-        __syncthreads();
-        block_sort_row<T>(sk, sv, N, val != nullptr);
-        for (int e = tid; e < len; e += nt) {
-            col[lo + e] = sk[e];
-            if (val) val[lo + e] = sv[e];
-        }
-        __syncthreads();
-    }
-}
-
-// ------------------------------------------- direct read into host memory
-//
-// Rows of C read straight into the caller's page-locked host buffers, which
-// the GPU reaches over the C2C link (out_col, out_val: their device
-// addresses), with one host synchronisation for the whole read.  Each warp
-// takes a row: a row of up to SORT_SHORT entries is put in column order in
-// registers (ranked by shuffles unless it is in order already) and written
-// out; a longer row is copied to device scratch at its place and listed for
-// k_long_rows_out.  Nothing is written when R is not the ordered list of its
-// collection (r_total != n) or the entries do not fit the caller's buffers;
-// the flags say which, and the caller takes the general path.
-template <typename T>
-__global__ void k_gather_sort_out(const int32_t *rows, int64_t n_arg, const long long *n_dev, MatView M,
-                                  const int64_t *rp, const int64_t *r_total, int64_t nnz_cap, int32_t *out_col,
-                                  T *out_val, int32_t *scr_col, T *scr_val, int64_t *long_list, ReadOut *res) {
-    pdl_begin();
-    const int64_t n = n_dev ? (int64_t)*n_dev : n_arg;
-    // rp[n] exists only when R was placed (r_total == n)
-    const bool unordered = r_total && *r_total != n;
-    const int64_t nnz = unordered ? 0 : rp[n];
-    const unsigned bad = (unordered ? READ_UNORDERED : 0u) | (nnz > nnz_cap ? READ_TOO_SMALL : 0u);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        res->nnz = nnz;
-        if (bad) atomicOr(&res->flags, bad);
-    }
-    if (bad) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const T *mv = (const T *)M.val;
-    for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < n; x += nwarps) {
-        const int64_t r = rows[x];
-        const int64_t so = M.off[r], d = rp[x];
-        const int L = M.len[r];
-        if (L <= SORT_SHORT) {
-            const int32_t k0 = lane < L ? M.col[so + lane] : INT32_MAX;
-            const int32_t k1 = lane + 32 < L ? M.col[so + lane + 32] : INT32_MAX;
-            T v0 = T(0), v1 = T(0);
-            if (out_val) {
-                if (lane < L) v0 = mv[so + lane];
-                if (lane + 32 < L) v1 = mv[so + lane + 32];
-            }
-            // entry e + 1 after entry e: the next lane's, across the halves at lane 31
-            const int32_t up0 = __shfl_down_sync(0xffffffffu, k0, 1);
-            const int32_t lo1 = __shfl_sync(0xffffffffu, k1, 0);
-            const int32_t up1 = __shfl_down_sync(0xffffffffu, k1, 1);
-            const int32_t n0 = lane == 31 ? lo1 : up0;
-            const bool out_of_order = (lane + 1 < L && k0 > n0) || (lane + 33 < L && k1 > up1);
-            int r0 = lane, r1 = lane + 32;
-            if (__any_sync(0xffffffffu, out_of_order)) {  // rank among the row's (distinct) columns
-                r0 = 0;
-                r1 = 0;
-                for (int j = 0; j < 32; j++) {
-                    const int32_t a = __shfl_sync(0xffffffffu, k0, j), b = __shfl_sync(0xffffffffu, k1, j);
-                    r0 += (a < k0) + (b < k0);
-                    r1 += (a < k1) + (b < k1);
-                }
-            }
-            if (lane < L) {
-                out_col[d + r0] = k0;
-                if (out_val) out_val[d + r0] = v0;
-            }
-            if (lane + 32 < L) {
-                out_col[d + r1] = k1;
-                if (out_val) out_val[d + r1] = v1;
-            }
-        } else {
-            for (int e = lane; e < L; e += 32) {
-                scr_col[d + e] = M.col[so + e];
-                if (out_val) scr_val[d + e] = mv[so + e];
-            }
-            if (lane == 0) long_list[atomicAdd(&res->n_long, 1u)] = x;
-        }
-    }
-}
-
-// The listed rows of more than SORT_SHORT entries, a block each: put in
-// column order in shared memory (unless in order already) and written from
-// the scratch to the caller's buffers; rows over SORT_MAX entries are listed
-// again (huge_list) and left for the host's radix sort of the scratch.
-template <typename T>
-__global__ void __launch_bounds__(512) k_long_rows_out(const int64_t *rp, const int64_t *long_list, const int32_t *scr_col,
-                                                       const T *scr_val, int32_t *out_col, T *out_val,
-                                                       int64_t *huge_list, ReadOut *res) {
+__global__ void __launch_bounds__(512)
+k_sort_long(const int32_t *rows, MatView M, const int64_t *rp, const int64_t *long_list, int32_t *dst_col, T *dst_val,
+            int32_t *out_col, T *out_val, bool has_val, int64_t *huge_list, ReadOut *res) {
     pdl_begin();
     extern __shared__ __align__(16) unsigned char smem[];
     T *sv = (T *)smem;
@@ -530,89 +661,85 @@ __global__ void __launch_bounds__(512) k_long_rows_out(const int64_t *rp, const 
     if (res->flags) return;
     const unsigned nl = res->n_long;
     const int tid = threadIdx.x, nt = blockDim.x;
+    const T *mv = (const T *)M.val;
+    int32_t *oc = out_col ? out_col : dst_col;
+    T *ov = out_col ? out_val : dst_val;
     for (unsigned j = blockIdx.x; j < nl; j += gridDim.x) {
         const int64_t x = long_list[j];
         const int64_t lo = rp[x];
         const int64_t len = rp[x + 1] - lo;
+        const int64_t so = M.off[rows ? (int64_t)rows[x] : x];
         int unsorted = 0;
-        for (int64_t e = tid; e + 1 < len; e += nt) unsorted |= scr_col[lo + e] > scr_col[lo + e + 1];
-        if (!__syncthreads_or(unsorted)) {
+        for (int64_t e = tid; e + 1 < len; e += nt) unsorted |= M.col[so + e] > M.col[so + e + 1];
+        const bool sort = __syncthreads_or(unsorted);
+        if (!sort || len > SORT_MAX) {
+            int32_t *tc = sort ? dst_col : oc;
+            T *tv = sort ? dst_val : ov;
             for (int64_t e = tid; e < len; e += nt) {
-                out_col[lo + e] = scr_col[lo + e];
-                if (out_val) out_val[lo + e] = scr_val[lo + e];
+                tc[lo + e] = M.col[so + e];
+                if (has_val) tv[lo + e] = mv[so + e];
             }
-            continue;
-        }
-        if (len > SORT_MAX) {
-            if (tid == 0) huge_list[atomicAdd(&res->n_huge, 1u)] = x;
+            if (sort && tid == 0) huge_list[atomicAdd(&res->n_huge, 1u)] = x;
             continue;
         }
         int N = 128;
         while (N < len) N <<= 1;
         for (int e = tid; e < N; e += nt) {
-            sk[e] = e < len ? scr_col[lo + e] : INT32_MAX;
-            if (out_val && e < len) sv[e] = scr_val[lo + e];
+            sk[e] = e < len ? M.col[so + e] : INT32_MAX;
+            if (has_val && e < len) sv[e] = mv[so + e];
         }
         __syncthreads();
-        block_sort_row<T>(sk, sv, N, out_val != nullptr);
+        block_sort_row<T>(sk, sv, N, has_val);
         for (int e = tid; e < len; e += nt) {
-            out_col[lo + e] = sk[e];
-            if (out_val) out_val[lo + e] = sv[e];
+            oc[lo + e] = sk[e];
+            if (has_val) ov[lo + e] = sv[e];
         }
         __syncthreads();
     }
 }
 
 template <typename T>
-static void read_rows_direct_t(const int32_t *rows, int64_t n, const long long *n_dev, const MatView &M,
-                               const int64_t *rp, const int64_t *r_total, int64_t nnz_cap, int32_t *out_col, T *out_val,
-                               int32_t *scr_col, T *scr_val, int64_t *long_list, int64_t *huge_list, ReadOut *res,
-                               cudaStream_t s, int num_sms) {
+static void read_rows_out_t(const int32_t *rows, int64_t n, const long long *n_dev, const MatView &M, bool has_val,
+                            const int64_t *rp, const int64_t *r_total, int64_t nnz_cap, int32_t *dst_col, T *dst_val,
+                            int32_t *out_col, T *out_val, int64_t *long_list, int64_t *huge_list, ReadOut *res,
+                            cudaStream_t s, int num_sms) {
     // n on the device: n is the host's bound on it, which sizes the grids
-    launch_k(k_gather_sort_out<T>, blocks_for(std::max<int64_t>(n, 1) * 32, 256, (int64_t)num_sms * 16), 256, 0, s, rows,
-             n, n_dev, M, rp, r_total, nnz_cap, out_col, out_val, scr_col, scr_val, long_list, res);
+    launch_k(k_read_short<T>, blocks_for(std::max<int64_t>(n, 1), RS_ROWS, (int64_t)num_sms * 8), RS_NT, 0, s, rows, n,
+             n_dev, M, rp, r_total, nnz_cap, out_col ? out_col : dst_col,
+             has_val ? (out_col ? out_val : dst_val) : (T *)nullptr, long_list, res);
+    if (M.ncols <= OL_MAX_COLS) {
+        const int W = (int)std::min<int64_t>(OL_W, std::max<int64_t>(1, (M.ncols + 1023) / 1024) * 1024);
+        const size_t smem = order_long_smem(W);
+        static bool set = false;
+        if (!set) {
+            cudaFuncSetAttribute(k_order_long<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)order_long_smem(OL_W));
+            set = true;
+        }
+        launch_k(k_order_long<T>, (unsigned)std::max<int64_t>(1, std::min<int64_t>(n, (int64_t)num_sms * 4)), OL_NT,
+                 smem, s, rows, M, rp, (const int64_t *)long_list, dst_col, dst_val, out_col, out_val, has_val, res, W);
+        return;
+    }
     const size_t smem = (size_t)SORT_MAX * (sizeof(T) + sizeof(int32_t));
     static bool set = false;
     if (!set) {
-        cudaFuncSetAttribute(k_long_rows_out<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(k_sort_long<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         set = true;
     }
-    launch_k(k_long_rows_out<T>, (unsigned)std::max<int64_t>(1, std::min<int64_t>(n, (int64_t)num_sms * 2)), 512, smem,
-             s, rp, long_list, scr_col, scr_val, out_col, out_val, huge_list, res);
+    launch_k(k_sort_long<T>, (unsigned)std::max<int64_t>(1, std::min<int64_t>(n, (int64_t)num_sms * 2)), 512, smem, s,
+             rows, M, rp, (const int64_t *)long_list, dst_col, dst_val, out_col, out_val, has_val, huge_list, res);
 }
 
-void read_rows_direct(const int32_t *rows, int64_t n, const long long *n_dev, const MatView &M, int vsize,
-                      const int64_t *rp, const int64_t *r_total, int64_t nnz_cap, int32_t *out_col, void *out_val,
-                      int32_t *scr_col, void *scr_val, int64_t *long_list, int64_t *huge_list, ReadOut *res,
-                      cudaStream_t s, int num_sms) {
+void read_rows_out(const int32_t *rows, int64_t n, const long long *n_dev, const MatView &M, int vsize,
+                   const int64_t *rp, const int64_t *r_total, int64_t nnz_cap, int32_t *dst_col, void *dst_val,
+                   int32_t *out_col, void *out_val, int64_t *long_list, int64_t *huge_list, ReadOut *res,
+                   cudaStream_t s, int num_sms) {
+    const bool has_val = vsize && M.val && (out_col ? out_val != nullptr : dst_val != nullptr);
     if (vsize == 8)
-        read_rows_direct_t<double>(rows, n, n_dev, M, rp, r_total, nnz_cap, out_col, (double *)out_val, scr_col,
-                                   (double *)scr_val, long_list, huge_list, res, s, num_sms);
+        read_rows_out_t<double>(rows, n, n_dev, M, has_val, rp, r_total, nnz_cap, dst_col, (double *)dst_val, out_col,
+                                (double *)out_val, long_list, huge_list, res, s, num_sms);
     else
-        read_rows_direct_t<int32_t>(rows, n, n_dev, M, rp, r_total, nnz_cap, out_col, (int32_t *)out_val, scr_col,
-                                    (int32_t *)scr_val, long_list, huge_list, res, s, num_sms);
-}
-
-template <typename T>
-static void sort_rows_t(const int64_t *rowptr, int64_t n, int32_t *col, T *val, unsigned *n_listed, int64_t *listed,
-                        int64_t list_cap, cudaStream_t s, int num_sms) {
-    launch_k(k_sort_short_rows<T>, blocks_for(n * 32, 256, (int64_t)num_sms * 16), 256, 0, s, rowptr, n, col, val);
-    const size_t smem = (size_t)SORT_MAX * (sizeof(T) + sizeof(int32_t));
-    static bool set = false;
-    if (!set) {
-        cudaFuncSetAttribute(k_sort_long_rows<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        set = true;
-    }
-    const int64_t g = std::min<int64_t>(n, (int64_t)num_sms * 2);
-    launch_k(k_sort_long_rows<T>, (unsigned)std::max<int64_t>(g, 1), 512, smem, s, rowptr, n, col, val, n_listed,
-             listed, list_cap);
-}
-
-void sort_rows(const int64_t *rowptr, int64_t n, int32_t *col, void *val, int vsize, unsigned *n_listed,
-               int64_t *listed, int64_t list_cap, cudaStream_t s, int num_sms) {
-    if (n <= 0 || !col) return;
-    if (vsize == 8) sort_rows_t<double>(rowptr, n, col, (double *)val, n_listed, listed, list_cap, s, num_sms);
-    else sort_rows_t<int32_t>(rowptr, n, col, (int32_t *)val, n_listed, listed, list_cap, s, num_sms);
+        read_rows_out_t<int32_t>(rows, n, n_dev, M, has_val, rp, r_total, nnz_cap, dst_col, (int32_t *)dst_val, out_col,
+                                 (int32_t *)out_val, long_list, huge_list, res, s, num_sms);
 }
 
 // Rows too long for a CTA's shared memory, sorted all at once: the packed

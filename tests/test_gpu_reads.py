@@ -1,0 +1,56 @@
+"""Rows of C read in column order, at the lengths and widths where the read's
+kernels change their way: 64 entries (a warp in registers, then a block with a
+bitmap), the bitmap's 1024-column stretches and 262144-column windows, and C
+wider than 2^22 columns (a sorting network, and the radix sort past 16384
+entries)."""
+
+import numpy as np
+import pytest
+
+from oracle import OMat
+from parity import assert_rows_match
+from workloads import CSR, MIN_PLUS_I32, PLUS_TIMES_F64
+
+pytestmark = pytest.mark.gpu
+
+LENGTHS = [0, 1, 31, 32, 33, 63, 64, 65, 66, 127, 128, 129, 511, 513, 1025, 2048, 16384, 16385, 20000]
+
+
+def _csr(rows, ncols, sr, rng):
+    rp = np.zeros(len(rows) + 1, np.int64)
+    np.cumsum([len(r) for r in rows], out=rp[1:])
+    col = np.concatenate([np.sort(r) for r in rows]).astype(np.int32) if rp[-1] else np.zeros(0, np.int32)
+    val = rng.random(col.shape[0]) if sr == PLUS_TIMES_F64 else rng.integers(1, 101, col.shape[0], dtype=np.int32)
+    return CSR(len(rows), ncols, rp, col, val)
+
+
+@pytest.mark.parametrize("sr", [PLUS_TIMES_F64, MIN_PLUS_I32])
+@pytest.mark.parametrize("m", [20480, (1 << 18), (1 << 18) + 1, 600001, (1 << 22) + 33])
+def test_rows_in_order_at_every_width(dspg, m, sr):
+    rng = np.random.default_rng(m + sr)
+    edges = np.array([c for c in (0, 1, 1023, 1024, (1 << 18) - 1, 1 << 18, (1 << 18) + 1, m - 2, m - 1) if c < m])
+    brows, arows = [], []
+    for length in LENGTHS:
+        cols = np.unique(np.concatenate([edges[: max(0, length // 8)], rng.choice(m, size=length, replace=False)]))
+        cols = rng.permutation(cols)[:length]
+        # each row of C is the union of disjoint rows of B, so that its columns arrive in runs
+        cut = np.array_split(cols, 3)
+        arows.append(np.arange(len(brows), len(brows) + 3))
+        brows += cut
+    arows.append(np.array([len(brows)]))
+    brows.append(rng.choice(m, size=5000, replace=False))  # one run: may leave its kernel in any order
+    A, B = _csr(arows, len(brows), sr, rng), _csr(brows, m, sr, rng)
+    g = dspg.DynamicSpGEMM(A, B)
+    Ao, Bo = OMat.from_csr(A), OMat.from_csr(B)
+    every = np.arange(A.nrows, dtype=np.int32)
+    orp, ocol, oval = Ao.multiply_rows(Bo, every)
+    sabs = Ao.multiply_rows(Bo, every, absval=True)[2] if sr == PLUS_TIMES_F64 else None
+    C = g.read_C()
+    assert_rows_match(C.rowptr, C.col, C.val, orp, ocol, oval, sabs, "host")
+    rp, col, val = (x.cpu().numpy() for x in g.read_C_device())
+    assert_rows_match(rp, col, val, orp, ocol, oval, sabs, "device")
+    pick = rng.permutation(every)[:9]  # rows in any order
+    orp, ocol, oval = Ao.multiply_rows(Bo, pick)
+    sabs = Ao.multiply_rows(Bo, pick, absval=True)[2] if sr == PLUS_TIMES_F64 else None
+    assert_rows_match(*g.read_rows_C(pick), orp, ocol, oval, sabs, "listed rows")
+    g.close()
