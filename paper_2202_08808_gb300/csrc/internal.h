@@ -354,8 +354,9 @@ struct dspg_estimator {
     float *master = nullptr;   // float32 parameters (device)
     float *grad = nullptr;     // last gradient (device)
     uint16_t *w = nullptr;     // bfloat16 bits of master (device)
-    float *H1 = nullptr, *H2 = nullptr, *D = nullptr, *DZ1 = nullptr, *DZ2 = nullptr, *O = nullptr;
-    int64_t cap = 0;           // rows the activation buffers hold
-    double *loss_d = nullptr;  // device accumulator
+    float *cols = nullptr;     // a step's activations and their gradients, a column per unit
+    int64_t cap = 0;           // rows they hold
+    double *lpart = nullptr;   // the blocks' squared errors
+    double *loss_d = nullptr;  // mean squared error
     std::string err;
 };
