@@ -26,9 +26,10 @@
 //     folded into Z(i,j) and sets bit k of H(i,j).
 //  5. Merge Z into C and H into F at C*'s entries (k_mask_plan,
 //     k_mask_splice): an entry of C* that received a product takes its new
-//     value and word (written in place, or appended when C had no entry
-//     there); one that received none leaves C (the row is compacted).
-//     Entries of C outside C* are not touched.
+//     value and word (written in place, or where C had no entry there, in
+//     the place of one that leaves or at the row's end); one that received
+//     none leaves C, and the row's last entries move into the places left.
+//     The other entries of C outside C* are not touched.
 //
 // Every k that contributes to an entry of C* at the end has its bit in E
 // (it contributed before, or one of its two factors changed), so A^R keeps
@@ -261,60 +262,161 @@ __global__ void k_pat_runs(MaskJob M, const int32_t *rflag, const int64_t *rex, 
 
 // --------------------------------------------------- E, R and A^R
 
-// A warp per run: each entry of the row of C is looked up in the run; a
-// hit records its place in the row and its word of F.  Then R_i = OR over
-// the run of (F | F*).
-__global__ void k_mask_scan(MaskJob M, MatView C, const unsigned long long *F) {
-    pdl_begin();
-    const int lane = threadIdx.x & 31;
-    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    const long long nr = *M.nruns_dev;
-    for (long long r = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < nr; r += nwarps) {
-        const int64_t u0 = M.run_start[r], u1 = M.run_start[r + 1];
-        const int32_t i = M.run_row[r];
-        const int64_t coff = C.off[i];
-        const int L = C.len[i];
-        for (int p = lane; p < L; p += 32) {
-            const int32_t j = C.col[coff + p];
-            const int64_t t = lower_bound_dev<int32_t>(M.ucol, u0, u1, j);
-            if (t < u1 && M.ucol[t] == j) {
-                M.upos[t] = p;
-                M.ue[t] = F[coff + p];
+// The entries of a row of C that are in its run of C*: their places and
+// words of F.  The row is read once, MS_U loads a thread in flight, and a
+// column goes on to the search of the run only when its bit of a filter of
+// the run's columns (nw words of shared memory, a bit per column) is set:
+// runs are a few entries long (2 on R-MAT with 1000 edges) and rows
+// thousands.  The nt threads t (a warp, or the block with BLOCK) share the row.
+constexpr int MS_NT = 256;
+constexpr int MS_U = 8;
+constexpr int MS_LONG = 2048;  // rows of more entries are read by the whole block (8192, with 4 loads in flight: 190 us)
+
+template <bool BLOCK>
+__device__ __forceinline__ void mask_scan_row(const MaskJob &M, const MatView &C, const unsigned long long *F, int64_t u0,
+                                              int64_t u1, int64_t coff, int L, uint32_t *filter, int lognw, int t) {
+    constexpr int NT = BLOCK ? MS_NT : 32;
+    auto sync = [&]() {
+        if (BLOCK) __syncthreads();
+        else __syncwarp();
+    };
+    const int shift = 32 - 5 - lognw;
+    for (int q = t; q < (1 << lognw); q += NT) filter[q] = 0u;
+    sync();
+    for (int64_t u = u0 + t; u < u1; u += NT) {
+        const uint32_t hsh = ((uint32_t)M.ucol[u] * 2654435761u) >> shift;
+        atomicOr(&filter[hsh >> 5], 1u << (hsh & 31));
+    }
+    sync();
+    for (int p0 = t; p0 < L; p0 += NT * MS_U) {
+        int32_t j[MS_U];
+#pragma unroll
+        for (int q = 0; q < MS_U; q++) j[q] = p0 + q * NT < L ? C.col[coff + p0 + q * NT] : -1;
+#pragma unroll
+        for (int q = 0; q < MS_U; q++) {
+            const uint32_t hsh = ((uint32_t)j[q] * 2654435761u) >> shift;
+            if (j[q] < 0 || !((filter[hsh >> 5] >> (hsh & 31)) & 1u)) continue;
+            const int64_t u = lower_bound_dev<int32_t>(M.ucol, u0, u1, j[q]);
+            if (u < u1 && M.ucol[u] == j[q]) {
+                M.upos[u] = p0 + q * NT;
+                M.ue[u] = F[coff + p0 + q * NT];
             }
         }
-        __syncwarp();
-        unsigned long long rb = 0;
-        for (int64_t t = u0 + lane; t < u1; t += 32) rb |= M.ue[t] | M.ufs[t];
-        rb = warp_or(rb);
-        if (lane == 0) M.rbits[r] = rb;
-        __syncwarp();
     }
+    sync();
 }
 
-// A warp per run: the entries of row i of A' whose bit is set in R_i.
-__global__ void k_mask_keep(MaskJob M, MatView A, Ctl *ctl) {
+// R_i = OR over the run of (F | F*), by a warp.
+__device__ __forceinline__ void mask_row_bits(const MaskJob &M, int64_t r, int64_t u0, int64_t u1, int lane) {
+    unsigned long long rb = 0;
+    for (int64_t u = u0 + lane; u < u1; u += 32) rb |= M.ue[u] | M.ufs[u];
+    rb = warp_or(rb);
+    if (lane == 0) M.rbits[r] = rb;
+}
+
+// A warp per run, the rows of more than MS_LONG entries by the whole block at
+// the end of its round.  Bound by the read of the rows (4 bytes an entry);
+// with a search per entry in global memory, a load after the other, the
+// kernel took 448 us on 1000 edges of R-MAT 17, 124 us now.
+__global__ void __launch_bounds__(MS_NT) k_mask_scan(MaskJob M, MatView C, const unsigned long long *F) {
     pdl_begin();
-    const int lane = threadIdx.x & 31;
-    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
+    __shared__ uint32_t s_filter[MS_NT / 32 * 32];
+    __shared__ long long s_long[MS_NT / 32];
+    __shared__ int s_nlong;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const long long nr = *M.nruns_dev;
-    for (long long r = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < nr; r += nwarps) {
-        const int32_t i = M.run_row[r];
-        const unsigned long long rb = M.rbits[r];
-        const int64_t aoff = A.off[i];
-        const int alen = A.len[i];
-        for (int q0 = 0; q0 < alen; q0 += 32) {
-            const int q = q0 + lane;
-            const bool keep = q < alen && ((rb & kbit(A.col[aoff + q])) != 0ull);
-            const long long t = warp_fetch_add(&ctl->mask_kept, keep ? 1 : 0);
-            if (keep) {
-                if (t < M.kcap) {
-                    M.kept_run[t] = (int32_t)r;
-                    M.kept_a[t] = aoff + q;
-                } else {
-                    set_status(ctl, ST_MASK_FULL);
-                }
+    for (long long r0 = (long long)blockIdx.x * (MS_NT / 32); r0 < nr; r0 += (long long)gridDim.x * (MS_NT / 32)) {
+        if (tid == 0) s_nlong = 0;
+        __syncthreads();
+        const long long r = r0 + w;
+        if (r < nr) {
+            const int64_t u0 = M.run_start[r], u1 = M.run_start[r + 1];
+            const int32_t i = M.run_row[r];
+            const int64_t coff = C.off[i];
+            const int L = C.len[i];
+            if (L > MS_LONG) {
+                if (lane == 0) s_long[atomicAdd(&s_nlong, 1)] = r;
+            } else {
+                mask_scan_row<false>(M, C, F, u0, u1, coff, L, s_filter + w * 32, 5, lane);
+                mask_row_bits(M, r, u0, u1, lane);
             }
         }
+        __syncthreads();
+        const int nl = s_nlong;
+        for (int q = 0; q < nl; q++) {
+            const long long rl = s_long[q];
+            const int64_t u0 = M.run_start[rl], u1 = M.run_start[rl + 1];
+            const int32_t i = M.run_row[rl];
+            mask_scan_row<true>(M, C, F, u0, u1, C.off[i], C.len[i], s_filter, 8, tid);
+            if (w == 0) mask_row_bits(M, rl, u0, u1, lane);
+        }
+        __syncthreads();
+    }
+}
+static_assert(MS_NT / 32 * 32 == 1 << 8, "the block's filter");
+
+// A warp per run: the entries of row i of A' whose bit is set in R_i.  They
+// are counted first, so that a block takes its runs' places with one atomic:
+// an atomic per 32 entries on the one counter took 414 us on 1000 edges of
+// R-MAT 17, 14 us now.
+constexpr int MK_U = 4;
+__global__ void __launch_bounds__(256) k_mask_keep(MaskJob M, MatView A, Ctl *ctl) {
+    pdl_begin();
+    __shared__ int s_n[8];
+    __shared__ long long s_base;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const long long nr = *M.nruns_dev;
+    for (long long r0 = (long long)blockIdx.x * 8; r0 < nr; r0 += (long long)gridDim.x * 8) {
+        const long long r = r0 + w;
+        unsigned long long rb = 0ull;
+        int64_t aoff = 0;
+        int alen = 0;
+        if (r < nr) {
+            const int32_t i = M.run_row[r];
+            rb = M.rbits[r];
+            aoff = A.off[i];
+            alen = A.len[i];
+        }
+        int n = 0;
+        for (int q0 = lane; q0 < alen; q0 += 32 * MK_U) {
+            int32_t k[MK_U];
+#pragma unroll
+            for (int q = 0; q < MK_U; q++) k[q] = q0 + 32 * q < alen ? A.col[aoff + q0 + 32 * q] : -1;
+#pragma unroll
+            for (int q = 0; q < MK_U; q++) n += k[q] >= 0 && (rb & kbit(k[q])) != 0ull;
+        }
+        n = warp_sum<int>(n);
+        if (lane == 0) s_n[w] = n;
+        __syncthreads();
+        if (tid == 0) {
+            int tot = 0;
+            for (int q = 0; q < 8; q++) {
+                const int v = s_n[q];
+                s_n[q] = tot;
+                tot += v;
+            }
+            s_base = tot ? (long long)atomicAdd((unsigned long long *)&ctl->mask_kept, (unsigned long long)tot) : 0;
+        }
+        __syncthreads();
+        long long t = s_base + s_n[w];
+        if (n > 0) {
+            for (int q0 = 0; q0 < alen; q0 += 32) {
+                const int q = q0 + lane;
+                const bool keep = q < alen && ((rb & kbit(A.col[aoff + q])) != 0ull);
+                const unsigned bal = __ballot_sync(0xffffffffu, keep);
+                const long long at = t + __popc(bal & lanemask_lt());
+                if (keep) {
+                    if (at < M.kcap) {
+                        M.kept_run[at] = (int32_t)r;
+                        M.kept_a[at] = aoff + q;
+                    } else {
+                        set_status(ctl, ST_MASK_FULL);
+                    }
+                }
+                t += __popc(bal);
+            }
+        }
+        __syncthreads();  // s_n and s_base are read before the next round writes them
     }
 }
 
@@ -411,9 +513,14 @@ __global__ void k_mask_plan(MaskJob M, MatView C, Ctl *ctl, unsigned mask, int s
 }
 
 // A warp per run: (moves the row to its new place first, when it has one)
-// writes the new values and words in place, removes the entries that
-// received no product (a compaction of the row in order), and appends the
-// new entries.
+// writes the new values and words in place.  The entries that received no
+// product leave holes: the new entries go into holes first, then to the
+// row's end, and when there are more holes than new entries, the row's last
+// entries move into the holes that remain (C's rows carry no column order).
+// So only the run and as many entries at the row's end are touched; the
+// compaction of the whole row in order that this replaces took 646 us on
+// 1000 edges of R-MAT 17, 25 us now.  The holes' places are listed in
+// the run's words ue, which are not needed any more.
 template <int SR>
 __global__ void k_mask_splice(MaskJob M, MatView C, unsigned long long *F, Ctl *ctl, unsigned mask) {
     pdl_begin();
@@ -440,61 +547,72 @@ __global__ void k_mask_splice(MaskJob M, MatView C, unsigned long long *F, Ctl *
             base = dest;
             __syncwarp();
         }
-        int ndel = 0;
-        for (int64_t u = u0 + lane; u < u1; u += 32) {
-            const int p = M.upos[u];
-            if (p < 0) continue;
-            if (M.hit[u]) {
+        unsigned long long *hole = M.ue + u0;  // the holes' places, in the run's order
+        int ndel = 0, nins = 0;
+        for (int64_t uc = u0; uc < u1; uc += 32) {
+            const int64_t u = uc + lane;
+            const int p = u < u1 ? M.upos[u] : -1;
+            const bool hit = u < u1 && M.hit[u] != 0;
+            const bool del = p >= 0 && !hit;
+            if (p >= 0 && hit) {
                 Cv[base + p] = z[u];
                 F[base + p] = M.h[u];
                 written++;
-            } else {
-                C.col[base + p] = -1;  // leaves the row below
-                ndel++;
+            }
+            const unsigned bd = __ballot_sync(0xffffffffu, del);
+            if (del) hole[ndel + __popc(bd & lanemask_lt())] = (unsigned long long)p;
+            ndel += __popc(bd);
+            nins += __popc(__ballot_sync(0xffffffffu, u < u1 && p < 0 && hit));
+        }
+        __syncwarp();
+        const int len = L - ndel + nins;
+        if (nins > 0) {
+            int m = 0;  // new entries placed
+            for (int64_t uc = u0; uc < u1; uc += 32) {
+                const int64_t u = uc + lane;
+                const bool ins = u < u1 && M.upos[u] < 0 && M.hit[u];
+                const unsigned bal = __ballot_sync(0xffffffffu, ins);
+                if (ins) {
+                    const int x = m + __popc(bal & lanemask_lt());
+                    const int d = x < ndel ? (int)hole[x] : L + x - ndel;
+                    C.col[base + d] = M.ucol[u];
+                    Cv[base + d] = z[u];
+                    F[base + d] = M.h[u];
+                    written++;
+                }
+                m += __popc(bal);
             }
         }
-        ndel = warp_sum<int>(ndel);
-        __syncwarp();
-        int len = L;
-        if (ndel > 0) {
-            // in order, chunk by chunk: a kept entry moves down to the count of
-            // kept entries before it, never above a place still to be read
-            int w = 0;
-            for (int p0 = 0; p0 < L; p0 += 32) {
+        if (ndel > nins) {
+            // the remaining holes: marked, and those below the new length
+            // listed again (a hole's new place in the list is never above its
+            // old one, and each round reads before it writes)
+            int nh = 0;
+            for (int x0 = nins; x0 < ndel; x0 += 32) {
+                const int x = x0 + lane;
+                const int p = x < ndel ? (int)hole[x] : INT32_MAX;
+                if (x < ndel) C.col[base + p] = -1;
+                const bool low = p < len;
+                const unsigned bal = __ballot_sync(0xffffffffu, low);
+                __syncwarp();
+                if (low) hole[nh + __popc(bal & lanemask_lt())] = (unsigned long long)p;
+                nh += __popc(bal);
+                __syncwarp();
+            }
+            // the entries past the new length that stay, one into each of them
+            int m = 0;
+            for (int p0 = len; p0 < L && m < nh; p0 += 32) {
                 const int p = p0 + lane;
                 const int32_t c = p < L ? C.col[base + p] : -1;
-                const bool keep = c >= 0;
-                T v = T(0);
-                unsigned long long f = 0ull;
-                if (keep) {
-                    v = Cv[base + p];
-                    f = F[base + p];
-                }
-                const unsigned bal = __ballot_sync(0xffffffffu, keep);
-                __syncwarp();
-                if (keep) {
-                    const int d = w + __popc(bal & lanemask_lt());
+                const unsigned bal = __ballot_sync(0xffffffffu, c >= 0);
+                if (c >= 0) {
+                    const int d = (int)hole[m + __popc(bal & lanemask_lt())];
                     C.col[base + d] = c;
-                    Cv[base + d] = v;
-                    F[base + d] = f;
+                    Cv[base + d] = Cv[base + p];
+                    F[base + d] = F[base + p];
                 }
-                w += __popc(bal);
-                __syncwarp();
+                m += __popc(bal);
             }
-            len = w;
-        }
-        for (int64_t u0c = u0; u0c < u1; u0c += 32) {
-            const int64_t u = u0c + lane;
-            const bool ins = u < u1 && M.upos[u] < 0 && M.hit[u];
-            const unsigned bal = __ballot_sync(0xffffffffu, ins);
-            if (ins) {
-                const int d = len + __popc(bal & lanemask_lt());
-                C.col[base + d] = M.ucol[u];
-                Cv[base + d] = z[u];
-                F[base + d] = M.h[u];
-                written++;
-            }
-            len += __popc(bal);
         }
         __syncwarp();
         if (lane == 0) {
