@@ -10,15 +10,18 @@
 //  * small batches (<= 8192 entries, key + index bits <= 64): one CTA does
 //    validation, key packing, all radix passes in shared memory, and the
 //    de-duplicating gather in a single launch;
-//  * larger batches: a key kernel, then per 8-bit digit a histogram kernel,
-//    a device scan of the digit counts, and a stable scatter kernel, then a
-//    gather kernel.
+//  * larger batches: a key kernel, then a launch per digit of at most 8 bits
+//    (k_radix_pass) while the tiles are few, beyond 2^20 entries a histogram
+//    kernel, a device scan of the digit counts and a stable scatter kernel
+//    per digit, then a gather kernel.
 //
 // Stable ranking inside a CTA: each warp owns a contiguous segment of the
 // tile and walks it 32 entries at a time; __match_any_sync groups lanes
 // with equal digits, the rank inside the group is a popcount, and a per-warp
 // shared-memory counter per digit carries ranks across rounds.  Per-digit
 // prefixes over warps (in warp order) then give each entry its position.
+#include <algorithm>
+
 #include <cooperative_groups.h>
 
 #include "common.cuh"
@@ -432,9 +435,196 @@ constexpr int MS_IPT = 8;
 constexpr int MS_TILE = MS_NT * MS_IPT;
 constexpr int MS_ROUNDS = MS_TILE / MS_NT;
 
+// ---- one launch per digit
+//
+// While a digit's counts over all tiles are few, every block of a pass
+// derives its own places from them, so a pass needs no histogram and no scan
+// launches: the pass before has counted, as it placed each key, the next
+// digit of the key in the tile it went to (an atomic per key, on nb x digits
+// counters).  A block reads the nb x digits counts (128 KB at most from L2)
+// while it ranks its keys.  Three count arrays take turns: read, counted up,
+// zeroed for the pass after the next.  On the 131072 launch size of a
+// 10^5-update stencil batch (42-bit keys, six passes) the sort takes 52
+// us; with a histogram, three scan launches and a scatter per digit it took
+// 143 us.  Past RP_MAX entries the counts a block reads outgrow the launches
+// saved.
+constexpr int RP_NT = 512;
+constexpr int RP_NW = RP_NT / 32;
+constexpr int RP_DIG = 256;
+constexpr int64_t RP_MAX = (int64_t)1 << 20;
+
+// keys per thread: tiles of 1024, 2048 or 4096 keys, so that up to 2^18 keys
+// spread over 64 to 128 blocks
+static int rp_ipt(int64_t n) { return n <= 65536 ? 2 : (n <= 262144 ? 4 : 8); }
+static int64_t rp_tiles(int64_t n) { return (n + (int64_t)rp_ipt(n) * RP_NT - 1) / ((int64_t)rp_ipt(n) * RP_NT); }
+
 void sort_tmp_sizes(int64_t n, int64_t *count_entries) {
     int64_t nb = (n + MS_TILE - 1) / MS_TILE;
     *count_entries = 256 * (nb > 0 ? nb : 1);
+    // the most tiles that any length up to n has
+    int64_t tiles = 1;
+    for (int64_t top : {(int64_t)65536, (int64_t)262144, RP_MAX}) tiles = std::max(tiles, rp_tiles(std::min(n, top)));
+    *count_entries = std::max(*count_entries, 3 * RP_DIG * tiles);
+}
+
+// The first pass's counts of a tile (row blockIdx.x of cnt), from the keys
+// kk of this thread (ok: real ones); the next pass's row is zeroed.
+template <int IPT>
+__device__ __forceinline__ void rp_first_counts(const uint64_t (&kk)[IPT], const bool (&ok)[IPT], int width, uint32_t *cnt,
+                                                uint32_t *cnt_next) {
+    __shared__ uint32_t h[RP_DIG];
+    if (threadIdx.x < RP_DIG) h[threadIdx.x] = 0u;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < IPT; r++)
+        if (ok[r]) atomicAdd(&h[kk[r] & ((1u << width) - 1u)], 1u);
+    __syncthreads();
+    if (threadIdx.x < RP_DIG) {
+        cnt[(int64_t)blockIdx.x * RP_DIG + threadIdx.x] = h[threadIdx.x];
+        cnt_next[(int64_t)blockIdx.x * RP_DIG + threadIdx.x] = 0u;
+    }
+}
+
+template <int IPT>
+__global__ void __launch_bounds__(RP_NT)
+k_radix_first(const uint64_t *k, int n, int width, uint32_t *cnt, uint32_t *cnt_next) {
+    pdl_begin();
+    uint64_t kk[IPT];
+    bool ok[IPT];
+#pragma unroll
+    for (int r = 0; r < IPT; r++) {
+        const int i = blockIdx.x * IPT * RP_NT + r * RP_NT + threadIdx.x;
+        ok[r] = i < n;
+        kk[r] = ok[r] ? k[i] : 0;
+    }
+    rp_first_counts<IPT>(kk, ok, width, cnt, cnt_next);
+}
+
+template <int IPT>
+__global__ void __launch_bounds__(RP_NT)
+k_radix_pass(const uint64_t *k, const uint32_t *v, int n, int shift, int width, int next_shift, int next_width,
+             const uint32_t *cnt, uint32_t *cnt_next, uint32_t *cnt_zero, int nb, uint64_t *k_out, uint32_t *v_out) {
+    pdl_begin();
+    constexpr int TILE = IPT * RP_NT;
+    __shared__ uint32_t wc[RP_NW * RP_DIG];  // per warp and digit: keys, then the keys of lower warps
+    __shared__ uint32_t s_all[RP_NT], s_low[RP_NT];
+    __shared__ uint32_t s_base[RP_DIG];      // first place of each digit's keys of this tile
+    __shared__ uint32_t s_w[RP_NW];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, me = blockIdx.x;
+    const int nd = 1 << width;
+    const int seg = me * TILE + w * 32 * IPT;
+    uint64_t kk[IPT];
+    uint32_t vv[IPT];
+#pragma unroll
+    for (int r = 0; r < IPT; r++) {
+        const int i = seg + r * 32 + lane;
+        kk[r] = i < n ? k[i] : 0;
+        vv[r] = i < n ? v[i] : 0u;
+    }
+    for (int d = tid; d < RP_NW * RP_DIG; d += RP_NT) wc[d] = 0u;
+    if (cnt_zero && tid < RP_DIG) cnt_zero[(int64_t)me * RP_DIG + tid] = 0u;
+    {
+        // digit d over the tiles: all keys, and those of lower tiles; with
+        // fewer digits than threads the tiles are shared out
+        const int d = tid & (nd - 1), part = tid >> width, parts = RP_NT >> width;
+        uint32_t all = 0, low = 0;
+#pragma unroll 16
+        for (int t = part; t < nb; t += parts) {
+            const uint32_t c = cnt[(int64_t)t * RP_DIG + d];
+            all += c;
+            low += t < me ? c : 0u;
+        }
+        s_all[tid] = all;
+        s_low[tid] = low;
+    }
+    __syncthreads();
+    uint32_t lr[IPT];
+    uint32_t *mine = wc + w * RP_DIG;
+#pragma unroll
+    for (int r = 0; r < IPT; r++) {
+        const bool ok = seg + r * 32 + lane < n;
+        const unsigned d = (unsigned)(kk[r] >> shift) & (unsigned)(nd - 1);
+        unsigned peers = __ballot_sync(0xffffffffu, ok);
+        if (!ok) peers = ~peers;
+#pragma unroll
+        for (int b = 0; b < 8; b++)
+            if (b < width) {
+                const bool bit = (d >> b) & 1u;
+                const unsigned bal = __ballot_sync(0xffffffffu, bit);
+                peers &= bit ? bal : ~bal;
+            }
+        const uint32_t before = mine[d];
+        __syncwarp();  // every lane has read the counter before the group's last lane bumps it
+        lr[r] = before + __popc(peers & lanemask_lt());
+        if (ok && lane == 31 - __clz(peers)) mine[d] = before + __popc(peers);
+        __syncwarp();
+    }
+    __syncthreads();
+    uint32_t all = 0, low = 0;
+    if (tid < nd) {
+        uint32_t s = 0;
+#pragma unroll
+        for (int ww = 0; ww < RP_NW; ww++) {
+            const uint32_t c = wc[ww * RP_DIG + tid];
+            wc[ww * RP_DIG + tid] = s;
+            s += c;
+        }
+        for (int q = tid; q < RP_NT; q += nd) {
+            all += s_all[q];
+            low += s_low[q];
+        }
+    }
+    const uint32_t incl = warp_incl_scan<uint32_t>(all);
+    if (lane == 31) s_w[w] = incl;
+    __syncthreads();
+    uint32_t off = 0;
+#pragma unroll
+    for (int ww = 0; ww < RP_NW; ww++) off += ww < w ? s_w[ww] : 0u;
+    if (tid < RP_DIG) s_base[tid] = off + incl - all + low;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < IPT; r++)
+        if (seg + r * 32 + lane < n) {
+            const unsigned d = (unsigned)(kk[r] >> shift) & (unsigned)(nd - 1);
+            const uint32_t pos = s_base[d] + mine[d] + lr[r];
+            k_out[pos] = kk[r];
+            v_out[pos] = vv[r];
+            if (cnt_next)
+                atomicAdd(&cnt_next[(int64_t)(pos / TILE) * RP_DIG + ((unsigned)(kk[r] >> next_shift) & ((1u << next_width) - 1u))],
+                          1u);
+        }
+}
+
+template <int IPT>
+static void rp_passes(uint64_t *k, uint32_t *v, uint64_t *k_alt, uint32_t *v_alt, int64_t n, int bits, uint32_t *counts,
+                      cudaStream_t s, bool *in_alt) {
+    const int nb = (int)rp_tiles(n);
+    const int passes = (bits + 7) / 8, width = (bits + passes - 1) / passes;
+    bool alt = false;
+    for (int p = 0; p < passes; p++) {
+        auto c = [&](int q) { return counts + (int64_t)(q % 3) * nb * RP_DIG; };
+        const bool more = p + 1 < passes;
+        launch_k(k_radix_pass<IPT>, nb, RP_NT, 0, s, (const uint64_t *)(alt ? k_alt : k), (const uint32_t *)(alt ? v_alt : v),
+                 (int)n, p * width, width, (p + 1) * width, width, (const uint32_t *)c(p), more ? c(p + 1) : (uint32_t *)nullptr,
+                 more ? c(p + 2) : (uint32_t *)nullptr, nb, alt ? k : k_alt, alt ? v : v_alt);
+        alt = !alt;
+    }
+    *in_alt = alt;
+}
+
+// digits of the first pass
+static int rp_width(int bits) { return (bits + (bits + 7) / 8 - 1) / ((bits + 7) / 8); }
+
+static void rp_sort(uint64_t *k, uint32_t *v, uint64_t *k_alt, uint32_t *v_alt, int64_t n, int bits, uint32_t *counts,
+                    bool counted, cudaStream_t s, bool *in_alt) {
+    const int nb = (int)rp_tiles(n), ipt = rp_ipt(n);
+    if (!counted) {
+        uint32_t *c0 = counts, *c1 = counts + (int64_t)nb * RP_DIG;
+        auto *first = ipt == 2 ? k_radix_first<2> : (ipt == 4 ? k_radix_first<4> : k_radix_first<8>);
+        launch_k(first, nb, RP_NT, 0, s, (const uint64_t *)k, (int)n, rp_width(bits), c0, c1);
+    }
+    auto *run = ipt == 2 ? rp_passes<2> : (ipt == 4 ? rp_passes<4> : rp_passes<8>);
+    run(k, v, k_alt, v_alt, n, bits, counts, s, in_alt);
 }
 
 __global__ void k_make_keys(const InArgs *in, int64_t n, int64_t nrows, int64_t ncols, int sr, bool check_values,
@@ -456,6 +646,56 @@ __global__ void k_make_keys(const InArgs *in, int64_t n, int64_t nrows, int64_t 
     if (!ok) set_status(ctl, ST_INVALID);
     k[i] = ok ? (((uint64_t)(uint32_t)r << cb) | (uint32_t)c) : 0;
     v[i] = (uint32_t)i;
+}
+
+// The same with the first pass's counts; the thread's entries are all loaded
+// before any is checked.  After a failed stage every key is padding, and
+// nothing reads the result.
+template <int IPT>
+__global__ void __launch_bounds__(RP_NT)
+k_make_keys_counted(const InArgs *in, int n, int64_t nrows, int64_t ncols, int sr, bool check_values, Ctl *ctl,
+                    unsigned skip_mask, int cb, uint64_t *k, uint32_t *v, int width, uint32_t *cnt, uint32_t *cnt_next) {
+    pdl_begin();
+    const InArgs a = *in;
+    // one answer for the block: a bit that another block sets meanwhile must not split it
+    const int m = __syncthreads_or(failed(ctl, skip_mask)) ? 0 : (int)a.n;
+    int32_t row[IPT], col[IPT];
+    uint8_t op[IPT];
+    bool fine[IPT];
+#pragma unroll
+    for (int r = 0; r < IPT; r++) {
+        const int i = blockIdx.x * IPT * RP_NT + r * RP_NT + threadIdx.x;
+        row[r] = i < m ? a.row[i] : 0;
+        col[r] = i < m ? a.col[i] : 0;
+        op[r] = i < m ? a.op[i] : (uint8_t)OP_DELETE;
+        fine[r] = true;
+        if (check_values && i < m) {
+            if (sr == SR_PT) fine[r] = isfinite(((const double *)a.val)[i]);
+            else {
+                const int32_t x = ((const int32_t *)a.val)[i];
+                fine[r] = x > -MP_LIMIT && x < MP_LIMIT;
+            }
+        }
+    }
+    uint64_t kk[IPT];
+    bool ok[IPT];
+#pragma unroll
+    for (int r = 0; r < IPT; r++) {
+        const int i = blockIdx.x * IPT * RP_NT + r * RP_NT + threadIdx.x;
+        ok[r] = i < n;
+        kk[r] = ~uint64_t(0);  // padding
+        if (i < m) {
+            const bool good = row[r] >= 0 && (int64_t)row[r] < nrows && col[r] >= 0 && (int64_t)col[r] < ncols &&
+                              op[r] <= OP_SET && (fine[r] || op[r] == OP_DELETE);
+            if (!good) set_status(ctl, ST_INVALID);
+            kk[r] = good ? (((uint64_t)(uint32_t)row[r] << cb) | (uint32_t)col[r]) : 0;
+        }
+        if (ok[r]) {
+            k[i] = kk[r];
+            v[i] = (uint32_t)i;
+        }
+    }
+    rp_first_counts<IPT>(kk, ok, width, cnt, cnt_next);
 }
 
 __global__ void __launch_bounds__(MS_NT)
@@ -538,6 +778,10 @@ __global__ void k_finalize(const uint64_t *k, const uint32_t *v, int64_t n, int 
 
 void radix_sort_pairs(uint64_t *k, uint32_t *v, uint64_t *k_alt, uint32_t *v_alt, int64_t n, int bits,
                       uint32_t *counts, int64_t *scan_tmp, int64_t *scan_out, cudaStream_t s, bool *in_alt) {
+    if (n <= RP_MAX && n > 0 && bits > 0) {
+        rp_sort(k, v, k_alt, v_alt, n, bits, counts, false, s, in_alt);
+        return;
+    }
     int64_t nb = (n + MS_TILE - 1) / MS_TILE;
     bool alt = false;
     for (int shift = 0; shift < bits; shift += 8) {
@@ -646,9 +890,17 @@ void sort_updates(const InArgs *in, int64_t n, int64_t nrows, int64_t ncols, int
         return;
     }
     unsigned nblk = (unsigned)((n + 255) / 256);
-    launch_k(k_make_keys, nblk, 256, 0, s, in, n, nrows, ncols, sr, check_values, ctl, skip_mask, cb, tmp.k0, tmp.i0);
     bool in_alt = false;
-    radix_sort_pairs(tmp.k0, tmp.i0, tmp.k1, tmp.i1, n, kb, tmp.counts, tmp.scan_tmp, tmp.scan_out, s, &in_alt);
+    if (n <= RP_MAX) {
+        const int ipt = rp_ipt(n), nb = (int)rp_tiles(n);
+        auto *keys = ipt == 2 ? k_make_keys_counted<2> : (ipt == 4 ? k_make_keys_counted<4> : k_make_keys_counted<8>);
+        launch_k(keys, nb, RP_NT, 0, s, in, (int)n, nrows, ncols, sr, check_values, ctl, skip_mask, cb, tmp.k0, tmp.i0,
+                 rp_width(kb), tmp.counts, tmp.counts + (int64_t)nb * RP_DIG);
+        rp_sort(tmp.k0, tmp.i0, tmp.k1, tmp.i1, n, kb, tmp.counts, true, s, &in_alt);
+    } else {
+        launch_k(k_make_keys, nblk, 256, 0, s, in, n, nrows, ncols, sr, check_values, ctl, skip_mask, cb, tmp.k0, tmp.i0);
+        radix_sort_pairs(tmp.k0, tmp.i0, tmp.k1, tmp.i1, n, kb, tmp.counts, tmp.scan_tmp, tmp.scan_out, s, &in_alt);
+    }
     launch_k(k_finalize, nblk, 256, 0, s, in_alt ? tmp.k1 : tmp.k0, in_alt ? tmp.i1 : tmp.i0, n, cb, in, sr, out, ctl,
                                     skip_mask);
 }
