@@ -1482,11 +1482,14 @@ k_num_cluster_hash(MatView A, MatView B, MatView C, CJob J, Ctl *ctl, unsigned e
 
 // ------------------------------------------------- global dense kernel
 
-// Up to this many mask words (512K columns) the read-out takes a thread per
-// mask word; wider rows go through the summary of touched words.
+// Up to this many mask words (512K columns) the row's mask lies in shared
+// memory (64 KB) and the read-out goes over all of it, a warp per 32 words,
+// 32 columns at a time: the accumulator is read and cleared in whole lines.
+// Wider rows keep the mask in global memory and go through the summary of
+// touched words.
 constexpr int GD_DIRECT = 16384;
 
-template <int SR>
+template <int SR, bool DIRECT>
 __global__ void __launch_bounds__(512)
 k_num_gdense(MatView A, MatView B, MatView C, CJob J, Ctl *ctl, unsigned mask, int bin) {
     pdl_begin();
@@ -1496,18 +1499,21 @@ k_num_gdense(MatView A, MatView B, MatView C, CJob J, Ctl *ctl, unsigned mask, i
     __shared__ int p_incl[512], p_blen[512], p_wsum[32];
     __shared__ int s_n;
     __shared__ long long s_dest;
+    extern __shared__ uint32_t gd_smem[];
     if (failed(ctl, mask)) return;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int nwords = (int)(J.gd_w / 32);
     const int nsum = (nwords + 31) / 32;
-    const bool direct = nwords <= GD_DIRECT;
     T *acc = (T *)J.gd_acc + (int64_t)blockIdx.x * J.gd_w;
-    uint32_t *msk = J.gd_mask + (int64_t)blockIdx.x * nwords;
+    uint32_t *msk = DIRECT ? gd_smem : J.gd_mask + (int64_t)blockIdx.x * nwords;
     uint32_t *sum = J.gd_sum + (int64_t)blockIdx.x * nsum;  // bit w: mask word w was touched
     T *Cv = (T *)C.val;
     BlockProdSmem<T> ps{p_boff, p_av, p_incl, p_blen, p_wsum};
     long long nnz_acc = 0;
     const long long cnt = ctl->bin_count[bin];
+    if (blockIdx.x >= cnt) return;  // no row for this CTA
+    if (DIRECT)  // the read-out of a row leaves the mask clear for the next
+        for (int q = tid; q < nwords; q += 512) msk[q] = 0u;
     for (long long it = blockIdx.x; it < cnt; it += gridDim.x) {
         int32_t i = J.bins[(int64_t)bin * J.bin_cap + it];
         if (!dcheck(ctl, i >= 0 && i < A.nrows, DBG_R_ROW, it)) i = 0;  // debug build: a bad list entry fails the batch
@@ -1516,49 +1522,69 @@ k_num_gdense(MatView A, MatView B, MatView C, CJob J, Ctl *ctl, unsigned mask, i
         block_products<SR>(A, B, i, ps, [&](int32_t j, T v) {
             // the product that sets the first bit of a mask word marks the
             // word in the summary, so the read-out skips untouched words
-            if (atomicOr(&msk[j >> 5], 1u << (j & 31)) == 0u && !direct)
+            if (atomicOr(&msk[j >> 5], 1u << (j & 31)) == 0u && !DIRECT)
                 atomicOr(&sum[j >> 10], 1u << ((j >> 5) & 31));
             Sr<SR>::acc(&acc[j], v);
         });
         __syncthreads();
-        if (direct) {
-            // few columns: a thread per mask word, in order (a block scan per
-            // 512 words gives each its offset); no summary needed
+        if constexpr (DIRECT) {
+            // few columns: each warp's stretch of the mask in order, after a
+            // block scan of the stretches' counts
+            const int per = ((nwords + 15) / 16 + 31) / 32 * 32;  // words of a warp (16 warps), in whole groups of 32
+            const int w0 = w * per, w1 = w0 + per < nwords ? w0 + per : nwords;
             int c = 0;
-            for (int wd = tid; wd < nwords; wd += 512) c += __popc(__ldcg(msk + wd));
+            for (int wd = w0 + lane; wd < w1; wd += 32) c += __popc(msk[wd]);
             c = warp_sum<int>(c);
-            if ((tid & 31) == 0 && c) atomicAdd(&s_n, c);
+            if (lane == 0) p_wsum[w] = c;
             __syncthreads();
-            const int n = s_n;
             if (tid == 0) {
+                int n = 0;
+                for (int q = 0; q < 16; q++) {
+                    const int v = p_wsum[q];
+                    p_wsum[q] = n;
+                    n += v;
+                }
+                s_n = n;
                 s_dest = c_row_dest(C, J, ctl, i, n);
                 nnz_acc += n;
             }
             __syncthreads();
             const long long dest = s_dest;
-            int run = 0;
-            for (int w0 = 0; w0 < nwords; w0 += 512) {
-                const int wd = w0 + tid;
-                uint32_t bits = wd < nwords ? __ldcg(msk + wd) : 0u;
-                const int e = __popc(bits);
-                const int incl = block_incl_scan(e, p_incl, p_wsum);
-                int o = run + p_incl[tid] - e;
-                if (bits) msk[wd] = 0u;
-                while (bits) {
-                    const int bt = __ffs(bits) - 1;
-                    bits &= bits - 1;
-                    const int j = (wd << 5) + bt;
-                    if (dest >= 0) {
-                        C.col[dest + o] = j;
-                        Cv[dest + o] = __ldcg(acc + j);
+            int o = p_wsum[w];
+            for (int wd0 = w0; wd0 < w1; wd0 += 32) {
+                const uint32_t word = wd0 + lane < w1 ? msk[wd0 + lane] : 0u;
+                if (wd0 + lane < w1) msk[wd0 + lane] = 0u;
+                unsigned some = __ballot_sync(0xffffffffu, word != 0u);
+                while (some) {  // two words at a time: their accumulator lines are in flight together
+                    const int q0 = __ffs(some) - 1;
+                    some &= some - 1;
+                    const int q1 = some ? __ffs(some) - 1 : -1;
+                    some &= some - 1;
+                    const uint32_t b0 = __shfl_sync(0xffffffffu, word, q0);
+                    const uint32_t b1 = q1 >= 0 ? __shfl_sync(0xffffffffu, word, q1 & 31) : 0u;
+                    const int j0 = ((wd0 + q0) << 5) + lane, j1 = ((wd0 + (q1 & 31)) << 5) + lane;
+                    const bool h0 = (b0 >> lane) & 1u, h1 = (b1 >> lane) & 1u;
+                    const T v0 = h0 ? __ldcg(acc + j0) : T(0), v1 = h1 ? __ldcg(acc + j1) : T(0);
+                    const int o0 = o + __popc(b0 & lanemask_lt()), o1 = o + __popc(b0) + __popc(b1 & lanemask_lt());
+                    if (h0) {
+                        if (dest >= 0) {
+                            C.col[dest + o0] = j0;
+                            Cv[dest + o0] = v0;
+                        }
+                        acc[j0] = Sr<SR>::zero();
                     }
-                    acc[j] = Sr<SR>::zero();
-                    o++;
+                    if (h1) {
+                        if (dest >= 0) {
+                            C.col[dest + o1] = j1;
+                            Cv[dest + o1] = v1;
+                        }
+                        acc[j1] = Sr<SR>::zero();
+                    }
+                    o += __popc(b0) + __popc(b1);
                 }
-                run += incl;
-                __syncthreads();
             }
-            if (tid == 0 && dest >= 0) C.len[i] = n;
+            if (tid == 0 && dest >= 0) C.len[i] = s_n;
+            __syncthreads();  // the mask is clear, and every thread has read s_dest and its offset
             continue;
         }
         // entries under summary word x (its touched mask words)
@@ -2117,22 +2143,37 @@ static void run_numeric_t(const MatView &A, const MatView &B, const MatView &C, 
         launch_s64();
         return;
     }
+    // the longest rows first: a kernel of few long rows leaves room on the
+    // SMs that the bins of shorter rows fill, and nothing long is left for
+    // the end (300-edge batches of R-MAT 18: the recompute 869 us with the
+    // global dense bin last, its mask in global memory, 732 so).  The global dense bin is always
+    // launched: rows of bins that are off go there.
+    {
+        const int64_t words = J.gd_w / 32;
+        const bool direct = words <= GD_DIRECT;
+        static bool set_g = false;
+        if (!set_g) {
+            cudaFuncSetAttribute(k_num_gdense<SR, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(GD_DIRECT * sizeof(uint32_t)));
+            set_g = true;
+        }
+        launch_k(direct ? k_num_gdense<SR, true> : k_num_gdense<SR, false>, grid_for(J.gd_ctas, J.rows_hint, 1), 512,
+                 direct ? (size_t)words * sizeof(uint32_t) : 0, next(), A, B, C, J, ctl, mask, (int)BIN_GD);
+    }
+    if (on(BIN_K8L)) launch_cluster_hash<SR, 14, 8>(A, B, C, J, ctl, mask, BIN_K8L, next(), num_sms);
+    if (on(BIN_K8)) launch_cluster_hash<SR, 13, 8>(A, B, C, J, ctl, mask, BIN_K8, next(), num_sms);
+    if (on(BIN_K4)) launch_cluster_hash<SR, 13, 4>(A, B, C, J, ctl, mask, BIN_K4, next(), num_sms);
+    if (on(BIN_K2)) launch_cluster_hash<SR, 13, 2>(A, B, C, J, ctl, mask, BIN_K2, next(), num_sms);
+    if (on(BIN_C16384)) launch_cta_hash<SR, 14>(A, B, C, J, ctl, mask, BIN_C16384, next(), num_sms);
+    if (on(BIN_C8192)) launch_cta_hash<SR, 13>(A, B, C, J, ctl, mask, BIN_C8192, next(), num_sms);
+    if (on(BIN_C4096)) launch_cta_hash<SR, 12>(A, B, C, J, ctl, mask, BIN_C4096, next(), num_sms);
+    if (on(BIN_C2048)) launch_cta_hash<SR, 11>(A, B, C, J, ctl, mask, BIN_C2048, next(), num_sms);
+    if (on(BIN_W1024)) launch_group_hash<SR, 10, 32, 4>(A, B, C, J, ctl, mask, BIN_W1024, next(), num_sms);
+    if (on(BIN_W512)) launch_group_hash<SR, 9, 32, 4>(A, B, C, J, ctl, mask, BIN_W512, next(), num_sms);
+    if (on(BIN_W256)) launch_group_hash<SR, 8, 32, 8>(A, B, C, J, ctl, mask, BIN_W256, next(), num_sms);
+    if (on(BIN_W128)) launch_group_hash<SR, 7, 32, 8>(A, B, C, J, ctl, mask, BIN_W128, next(), num_sms);
     if (on(BIN_G16)) launch_group_hash<SR, 6, 16, 8>(A, B, C, J, ctl, mask, BIN_G16, next(), num_sms);
     if (on(BIN_G8)) launch_group_hash<SR, 5, 8, 8>(A, B, C, J, ctl, mask, BIN_G8, next(), num_sms);
-    if (on(BIN_W128)) launch_group_hash<SR, 7, 32, 8>(A, B, C, J, ctl, mask, BIN_W128, next(), num_sms);
-    if (on(BIN_W256)) launch_group_hash<SR, 8, 32, 8>(A, B, C, J, ctl, mask, BIN_W256, next(), num_sms);
-    if (on(BIN_W512)) launch_group_hash<SR, 9, 32, 4>(A, B, C, J, ctl, mask, BIN_W512, next(), num_sms);
-    if (on(BIN_W1024)) launch_group_hash<SR, 10, 32, 4>(A, B, C, J, ctl, mask, BIN_W1024, next(), num_sms);
-    if (on(BIN_C2048)) launch_cta_hash<SR, 11>(A, B, C, J, ctl, mask, BIN_C2048, next(), num_sms);
-    if (on(BIN_C4096)) launch_cta_hash<SR, 12>(A, B, C, J, ctl, mask, BIN_C4096, next(), num_sms);
-    if (on(BIN_C8192)) launch_cta_hash<SR, 13>(A, B, C, J, ctl, mask, BIN_C8192, next(), num_sms);
-    if (on(BIN_C16384)) launch_cta_hash<SR, 14>(A, B, C, J, ctl, mask, BIN_C16384, next(), num_sms);
-    if (on(BIN_K2)) launch_cluster_hash<SR, 13, 2>(A, B, C, J, ctl, mask, BIN_K2, next(), num_sms);
-    if (on(BIN_K4)) launch_cluster_hash<SR, 13, 4>(A, B, C, J, ctl, mask, BIN_K4, next(), num_sms);
-    if (on(BIN_K8)) launch_cluster_hash<SR, 13, 8>(A, B, C, J, ctl, mask, BIN_K8, next(), num_sms);
-    if (on(BIN_K8L)) launch_cluster_hash<SR, 14, 8>(A, B, C, J, ctl, mask, BIN_K8L, next(), num_sms);
-    // the global dense bin is always launched: rows of bins that are off go there
-    launch_k(k_num_gdense<SR>, grid_for(J.gd_ctas, J.rows_hint, 1), 512, 0, next(), A, B, C, J, ctl, mask, (int)BIN_GD);
     launch_s64();
 }
 
