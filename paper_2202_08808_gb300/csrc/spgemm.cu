@@ -192,7 +192,8 @@ constexpr int SIZE_SHORT = 64;   // A rows up to this length are sized by one th
 constexpr int SIZE_LONG = 512;   // up to this by a warp, longer ones by the whole block
 constexpr long long SPLIT_MIN = 8192;  // dense mode: rows with more products, or with more than
 constexpr int SPLIT_A = 256;           // SPLIT_A A entries, are split in chunks (k_num_dsplit)
-constexpr int SPLIT_CHUNK = 2048;      // A entries per work item of a split row
+constexpr int SPLIT_CHUNK = 256;       // A entries per work item of a split row: a round of the block's warps
+constexpr int SPLIT_END = 2;           // units of the work list after a row's chunks, for the work at its end
 constexpr int DS_NT = 256;             // threads of a split-kernel block
 
 // Dense mode: claim a split slot for a row with very many products; false
@@ -1803,10 +1804,24 @@ void run_size_bins(const MatView &A, const MatView &B, const MatView &C, const C
 // Dense mode, rows with many A entries or products (the hubs of skewed
 // graphs): each split row is cut into chunks of SPLIT_CHUNK A entries, and
 // the chunks of all split rows form one work list (k_split_prep writes its
-// prefix over the rows, sp_pre).  A CTA accumulates a chunk in shared memory
-// and folds it into the row's global accumulator with atomics; the CTA that
-// folds a row's last chunk (a per-row counter) writes the row into C in
-// column order and resets the accumulator for the next launch.
+// prefix over the rows, sp_pre; SPLIT_END units more per row stand for
+// writing it).  A CTA takes an equal, contiguous share of the list and
+// accumulates a row's chunks in it in shared memory.  A row that is all its
+// own it writes from there; of others it folds its part into the row's
+// global accumulator with atomics, and the CTA that folds the last chunk (a
+// per-row counter) writes the row into C in column order and resets the
+// accumulator for the next launch.
+// Bound by the gathers of B's row headers and entries (a few per row) from
+// L2.  A warp runs three steps ahead of itself, so that a step waits for one
+// of the three loads that follow one another instead of all of them:
+// the A entries of step t + 2, the B headers of step t + 1 and the B entries
+// of step t are in flight together.  Columns present need no atomic: in
+// (min,+) an accumulator that is not the neutral element has been reached (a
+// sum of two values below 2^30 is never INT32_MAX), in (+,.) a byte is
+// stored.  1000 edges of R-MAT 20 against 256 columns (3.5 million A
+// entries): 132 us with chunks of 2048 entries, the loads one after the other
+// an atomic per product on the presence words and every row folded through
+// global memory, 80 us now (SPLIT_END 2 to 16: 316, 320, 329, 337 us a pass).
 __global__ void __launch_bounds__(1024) k_split_prep(MatView A, CJob J, Ctl *ctl, unsigned mask) {
     pdl_begin();
     __shared__ int incl[1024], wsum[32];
@@ -1819,7 +1834,7 @@ __global__ void __launch_bounds__(1024) k_split_prep(MatView A, CJob J, Ctl *ctl
         int nch = 0;
         if (slot < cnt) {
             const int32_t i = J.bins[(int64_t)BIN_DSPLIT * J.bin_cap + slot];
-            nch = (A.len[i] + SPLIT_CHUNK - 1) / SPLIT_CHUNK;
+            nch = (A.len[i] + SPLIT_CHUNK - 1) / SPLIT_CHUNK + SPLIT_END;
         }
         const int tot = block_incl_scan(nch, incl, wsum);
         if (slot < cnt) J.sp_pre[slot] = carry + incl[threadIdx.x] - nch;
@@ -1827,6 +1842,78 @@ __global__ void __launch_bounds__(1024) k_split_prep(MatView A, CJob J, Ctl *ctl
         __syncthreads();
     }
     if (threadIdx.x == 0) J.sp_pre[cnt] = carry;
+}
+
+// Calls emit(j, a (x) b) for the products of the A entries [a_lo, a_hi) of
+// the row at aoff, this warp taking the groups of 32 from w * 32 in steps of
+// NT; returns the products of this lane's A entries.
+template <int SR, int NT, class F>
+__device__ __forceinline__ long long split_products(const MatView &A, const MatView &B, int64_t aoff, int a_lo, int a_hi,
+                                                    F emit) {
+    using T = typename Sr<SR>::T;
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const T *Av = (const T *)A.val;
+    const T *Bv = (const T *)B.val;
+    const int first = a_lo + (threadIdx.x >> 5) * 32 + lane;
+    long long prods = 0;
+    // in flight: the A entry of the step after the next (k2, av2), and the next step's B header
+    auto load_a = [&](int ai, int32_t &k, T &av) {
+        k = ai < a_hi ? A.col[aoff + ai] : -1;
+        av = ai < a_hi ? Av[aoff + ai] : T(0);
+    };
+    auto load_b = [&](int32_t k, int64_t &off, int &len) {
+        off = k >= 0 ? B.off[k] : 0;
+        len = k >= 0 ? B.len[k] : 0;
+    };
+    int32_t k1, k2;
+    T av1, av2;
+    load_a(first, k1, av1);
+    load_a(first + NT, k2, av2);
+    int64_t boff;
+    int blen;
+    load_b(k1, boff, blen);
+    for (int ai = first; ai - lane < a_hi; ai += NT) {
+        const T av = av1;
+        const int64_t bo = boff;
+        const int bl = blen;
+        k1 = k2;
+        av1 = av2;
+        load_a(ai + 2 * NT, k2, av2);
+        load_b(k1, boff, blen);
+        prods += bl;
+        int incl = bl;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int o = __shfl_up_sync(FULL, incl, d);
+            if (lane >= d) incl += o;
+        }
+        const int total = __shfl_sync(FULL, incl, 31);
+        const int64_t rel = bo - (incl - bl);  // product p of this lane's entry is B entry rel + p
+        for (int base = 0; base < total; base += 32 * PU) {
+            int32_t c[PU];
+            T v[PU], a[PU];
+#pragma unroll
+            for (int u = 0; u < PU; u++) {
+                const int p = base + u * 32 + lane;
+                int s = 0;
+#pragma unroll
+                for (int step = 16; step > 0; step >>= 1)
+                    if (__shfl_sync(FULL, incl, s + step - 1) <= p) s += step;
+                const int64_t q = __shfl_sync(FULL, rel, s) + p;
+                a[u] = __shfl_sync(FULL, av, s);
+                c[u] = -1;
+                if (p < total) {
+                    c[u] = __ldg(B.col + q);
+                    v[u] = __ldg(Bv + q);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < PU; u++)
+                if (c[u] >= 0) emit(c[u], Sr<SR>::mul(a[u], v[u]));
+        }
+    }
+    return prods;
 }
 
 template <int SR, int NT>
@@ -1837,23 +1924,26 @@ k_num_dsplit(MatView A, MatView B, MatView C, CJob J, Ctl *ctl, unsigned mask, i
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_last;
     __shared__ long long s_dest;
-    __shared__ int s_n;
+    __shared__ uint32_t s_word[32];  // the row's presence words, and the entries before each
+    __shared__ int s_off[32];
     if (failed(ctl, mask)) return;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31;
     const int nw = mp >> 5;
     T *acc = (T *)smem;
-    uint32_t *msk = (uint32_t *)(acc + mp);
+    uint8_t *pres = (uint8_t *)(acc + mp);  // (+,.): column reached
     T *Cv = (T *)C.val;
-    for (int s = tid; s < mp; s += NT) acc[s] = Sr<SR>::zero();
-    if (tid < 32) msk[tid] = 0u;
+    for (int s = tid; s < mp; s += NT) {
+        acc[s] = Sr<SR>::zero();
+        if (SR == SR_PT) pres[s] = 0;
+    }
     __syncthreads();
     long long cnt = ctl->bin_count[BIN_DSPLIT];
     if (cnt > J.sp_rows) cnt = J.sp_rows;
     const long long total = cnt > 0 ? J.sp_pre[cnt] : 0;
     long long nnz_acc = 0;
     // each CTA takes a contiguous range of work items: one search for its
-    // first row, then forward; consecutive chunks of a row are accumulated
-    // together and folded once
+    // first row, then forward; its chunks of a row are accumulated together
+    // and folded once
     const long long per = (total + gridDim.x - 1) / gridDim.x;
     const long long w0 = (long long)blockIdx.x * per, w1 = w0 + per < total ? w0 + per : total;
     long long slot = 0;
@@ -1865,86 +1955,98 @@ k_num_dsplit(MatView A, MatView B, MatView C, CJob J, Ctl *ctl, unsigned mask, i
         }
         slot = lo;
     }
-    int pending = 0;  // chunks accumulated in shared memory, not yet folded
     long long prods = 0;  // products formed (the sizing pass does not sum split rows)
-    for (long long w = w0; w < w1; w++) {
-        while (J.sp_pre[slot + 1] <= w) slot++;
-        const long long base = J.sp_pre[slot];
-        const int nch = (int)(J.sp_pre[slot + 1] - base);
-        const int c = (int)(w - base);
+    for (long long w = w0; w < w1; slot++) {
+        const long long base = J.sp_pre[slot], next = J.sp_pre[slot + 1];
         const int32_t i = J.bins[(int64_t)BIN_DSPLIT * J.bin_cap + slot];
         const int alen = A.len[i];
-        const int a_lo = c * SPLIT_CHUNK, a_hi = a_lo + SPLIT_CHUNK < alen ? a_lo + SPLIT_CHUNK : alen;
-        // each warp takes groups of 32 A entries of the chunk (no block barriers)
-        group_products<SR, 32>(A, B, i, 0xffffffffu, [&](int32_t j, T v) {
-            atomicOr(&msk[j >> 5], 1u << (j & 31));
-            Sr<SR>::acc(&acc[j], v);
-            prods++;
-        }, a_lo + (tid >> 5) * 32, a_hi, NT);
-        pending++;
-        if (c + 1 < nch && w + 1 < w1) continue;  // the next item is this row's next chunk: keep accumulating
+        const int nch = (alen + SPLIT_CHUNK - 1) / SPLIT_CHUNK;
+        const int c0 = (int)(w - base);
+        const long long end = next < w1 ? next : w1;
+        const int c1 = end - base < nch ? (int)(end - base) : nch;
+        w = end;
+        if (c0 >= c1) continue;  // only units that stand for the row's end
+        const int pending = c1 - c0;  // this CTA's chunks of the row
+        prods += split_products<SR, NT>(A, B, A.off[i], c0 * SPLIT_CHUNK, c1 == nch ? alen : c1 * SPLIT_CHUNK,
+                                        [&](int32_t j, T v) {
+                                            if (SR == SR_PT) pres[j] = 1;
+                                            Sr<SR>::acc(&acc[j], v);
+                                        });
         __syncthreads();
+        const bool whole = pending == nch;  // nobody else has a part of this row
         T *gacc = (T *)J.sp_acc + slot * mp;
         uint32_t *gmsk = J.sp_mask + slot * nw;
-        // fold: each present column into the global row, each mask word once;
-        // then one barrier, the mask reset and the row's chunk counter
+        // each present column into the row's global accumulator (mp is a
+        // multiple of 32: a warp is in or out as a whole); a whole row only
+        // needs its presence words
         for (int j = tid; j < mp; j += NT) {
-            const uint32_t word = msk[j >> 5];
-            if ((j & 31) == 0 && word) atomicOr(&gmsk[j >> 5], word);
-            if (word & (1u << (j & 31))) {
-                Sr<SR>::acc(&gacc[j], acc[j]);
+            const T v = acc[j];
+            const bool has = SR == SR_PT ? pres[j] != 0 : v != Sr<SR>::zero();
+            const uint32_t word = __ballot_sync(0xffffffffu, has);
+            if (whole) {
+                if (lane == 0) s_word[j >> 5] = word;
+                continue;
+            }
+            if (lane == 0 && word) atomicOr(&gmsk[j >> 5], word);
+            if (has) {
+                Sr<SR>::acc(&gacc[j], v);
                 acc[j] = Sr<SR>::zero();
+                if (SR == SR_PT) pres[j] = 0;
             }
         }
-        __threadfence();
-        __syncthreads();
-        if (tid < 32) msk[tid] = 0u;
-        if (tid == 0) s_last = atomicAdd(&J.sp_done[slot], pending) == nch - pending;
-        pending = 0;
-        __syncthreads();
-        if (s_last) {  // every chunk of the row is folded: write the row
+        if (!whole) {
             __threadfence();
-            if (tid < 32) {
-                const int lane = tid;
-                const uint32_t word = lane < nw ? __ldcg(gmsk + lane) : 0u;
-                const int pc = __popc(word);
-                const int incl = warp_incl_scan<int>(pc);
-                const int n = __shfl_sync(0xffffffffu, incl, 31);
-                int64_t dest = 0;
-                if (lane == 0) dest = c_row_dest(C, J, ctl, i, n);
-                dest = __shfl_sync(0xffffffffu, dest, 0);
-                int o = incl - pc;
-                uint32_t bits = word;
-                while (bits) {
-                    const int b = __ffs(bits) - 1;
-                    bits &= bits - 1;
-                    const int j = (lane << 5) + b;
-                    if (dest >= 0) {
-                        C.col[dest + o] = j;
-                        Cv[dest + o] = __ldcg(gacc + j);
-                    }
-                    o++;
-                }
-                if (lane == 0) {
-                    s_dest = dest;
-                    s_n = n;
-                }
-            }
             __syncthreads();
-            for (int j = tid; j < mp; j += NT) gacc[j] = Sr<SR>::zero();
-            if (tid < nw) gmsk[tid] = 0u;
-            if (tid == 0) {
-                if (s_dest >= 0) C.len[i] = s_n;
-                nnz_acc += s_n;
-                J.sp_done[slot] = 0;
+            if (tid == 0) s_last = atomicAdd(&J.sp_done[slot], pending) == nch - pending;
+            __syncthreads();
+            if (!s_last) continue;  // uniform; the next writes to s_last follow a barrier
+            __threadfence();
+            if (tid < nw) s_word[tid] = __ldcg(gmsk + tid);
+        }
+        __syncthreads();
+        // the row is complete: place it, then write it in column order and
+        // reset the accumulator it came from
+        if (tid < 32) {
+            const int pc = lane < nw ? __popc(s_word[lane]) : 0;
+            const int incl = warp_incl_scan<int>(pc);
+            s_off[lane] = incl - pc;
+            const int n = __shfl_sync(0xffffffffu, incl, 31);
+            if (lane == 0) {
+                const int64_t dest = c_row_dest(C, J, ctl, i, n);
+                s_dest = dest;
+                if (dest >= 0) C.len[i] = n;
+                nnz_acc += n;
             }
         }
         __syncthreads();
+        const long long dest = s_dest;
+        for (int j = tid; j < mp; j += NT) {
+            const uint32_t word = s_word[j >> 5];
+            if ((word >> lane) & 1u) {
+                if (dest >= 0) {
+                    const int o = s_off[j >> 5] + __popc(word & lanemask_lt());
+                    C.col[dest + o] = j;
+                    Cv[dest + o] = whole ? acc[j] : __ldcg(gacc + j);
+                }
+                if (whole) {
+                    acc[j] = Sr<SR>::zero();
+                    if (SR == SR_PT) pres[j] = 0;
+                } else {
+                    gacc[j] = Sr<SR>::zero();
+                }
+            }
+        }
+        if (!whole) {
+            if (tid < nw) gmsk[tid] = 0u;
+            if (tid == 0) J.sp_done[slot] = 0;
+        }
+        __syncthreads();  // the accumulator is clear, and s_word, s_off and s_dest are read
     }
     prods = warp_sum<long long>(prods);
-    if ((tid & 31) == 0 && prods && !J.count_only) atomic_add_ll2(&ctl->products, prods);
+    if (lane == 0 && prods && !J.count_only) atomic_add_ll2(&ctl->products, prods);
     if (tid == 0 && nnz_acc) atomic_add_ll2(&ctl->nnz_written, nnz_acc);
 }
+static_assert(SPLIT_CHUNK % DS_NT == 0 || DS_NT % SPLIT_CHUNK == 0, "a chunk is a whole number of the block's rounds, or less than one");
 
 // A persistent grid of `full` blocks, but no more blocks than it takes for
 // `rows` rows at `per_block` rows per block (small matrices launch small).
@@ -2137,8 +2239,8 @@ static void run_numeric_t(const MatView &A, const MatView &B, const MatView &C, 
             const unsigned early = mask & (ST_INVALID | ST_AB_STAGE | ST_AB_ARENA);
             launch_k(k_split_prep, 1, 1024, 0, ss, A, J, ctl, early);
             // blocks of DS_NT threads, 1024 threads an SM: a row's fold waits for fewer warps
-            launch_k(k_num_dsplit<SR, DS_NT>, (unsigned)((1024 / DS_NT) * num_sms), DS_NT, smem_c, ss, A, B, C, J,
-                     ctl, early, mp);
+            launch_k(k_num_dsplit<SR, DS_NT>, (unsigned)((1024 / DS_NT) * num_sms), DS_NT,
+                     (size_t)mp * (sizeof(T) + (SR == SR_PT ? 1 : 0)), ss, A, B, C, J, ctl, early, mp);
         }
         launch_s64();
         return;
