@@ -441,6 +441,7 @@ struct dspg_handle {
     uint64_t c_serial = 0;
     struct ReadKey {
         bool valid = false;
+        bool all = false;  // every row of C
         uint64_t serial = 0;
         int64_t nnz = 0;
         std::vector<int32_t> rows;
@@ -1445,18 +1446,21 @@ int64_t read_mat(dspg_handle *h, DevMat &M, const int32_t *rows_in, int64_t nr, 
     const int32_t *rows = nullptr;
     int64_t n = M.nrows;
     if (rows_in) n = nr;
-    // host rows of C that the last read of this generation of C listed too:
-    // their row pointers are still in the kept buffer
+    // the fill call of a two-call read of C: the row pointers of its count
+    // call, of the same generation of C and the same rows (host rows listed
+    // again, or all of them), are still in the kept buffer
     dspg_handle::ReadKey &key = h->rd_key;
-    const bool keyed = rows_in && !on_device && &M == &h->C;
-    const bool hit = keyed && key.valid && key.serial == h->c_serial && (int64_t)key.rows.size() == n &&
-                     (n == 0 || std::memcmp(key.rows.data(), rows_in, sizeof(int32_t) * (size_t)n) == 0);
+    const bool keyed = &M == &h->C && (!rows_in || !on_device);
+    const bool hit = keyed && key.valid && key.serial == h->c_serial && key.all == !rows_in &&
+                     (rows_in ? (int64_t)key.rows.size() == n &&
+                                    (n == 0 || std::memcmp(key.rows.data(), rows_in, sizeof(int32_t) * (size_t)n) == 0)
+                              : rowptr != nullptr);
     key.valid = false;  // the kept row list and row pointers are rewritten below unless this is a hit
     DBuf<int64_t> rp_l;
     int64_t *rp;
     int64_t nnz;
     if (hit) {
-        rows = h->rd.rows.p;
+        rows = rows_in ? h->rd.rows.p : nullptr;  // every row: no list
         rp = h->rd.rp.p;
         nnz = key.nnz;
     } else {
@@ -1471,8 +1475,9 @@ int64_t read_mat(dspg_handle *h, DevMat &M, const int32_t *rows_in, int64_t nr, 
         rp = read_scratch(h->rd.rp, rp_l, n + 1);
         nnz = mat_rowptr(h, M, rows, n, rp, s);
     }
-    if (keyed && rows == h->rd.rows.p && rp == h->rd.rp.p) {
-        if (!hit) key.rows.assign(rows_in, rows_in + n);
+    if (keyed && rp == h->rd.rp.p && (rows_in ? rows == h->rd.rows.p : !rowptr)) {
+        if (rows_in && !hit) key.rows.assign(rows_in, rows_in + n);
+        key.all = !rows_in;
         key.serial = h->c_serial;
         key.nnz = nnz;
         key.valid = true;
@@ -2579,6 +2584,7 @@ dspg_status dspg_read_affected_C(dspg_handle *h, int64_t rows_cap, int64_t nnz_c
         dspg_handle::ReadWs &w = h->rd;
         w.r.reserve(std::max<int64_t>(n, 1));
         DBuf<int64_t> rp_l;
+        h->rd_key.valid = false;  // the kept row pointers are rewritten
         int64_t *rp = read_scratch(w.rp, rp_l, n + 1);
         // R in row order on the device, from the chunk table of its collection
         const int64_t nch = ((h->A.nrows + 31) / 32 + 255) / 256;
@@ -2701,6 +2707,7 @@ dspg_status dspg_apply_read_affected(dspg_handle *h, const dspg_updates *dA, con
             const int64_t rc = std::max<int64_t>(cap, 1);
             w.r.reserve(rc);
             w.lens.reserve(rc);
+            h->rd_key.valid = false;  // the kept row pointers are rewritten
             w.rp.reserve(rc + 1);
             w.chunk_cnt.reserve(nch + 1);
             w.chunk_ex.reserve(nch + 1);

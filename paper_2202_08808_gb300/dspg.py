@@ -334,6 +334,9 @@ class DynamicSpGEMM:
         if st != 0:
             raise DspgError(st, self._lib.dspg_last_error(None).decode())
         self.b_is_a = B is None
+        d = [C.c_int64() for _ in range(3)]
+        self._check(self._lib.dspg_info(self._h, *[C.byref(x) for x in d], None, None))
+        self._n, _, self._m = (x.value for x in d)  # C's shape, which never changes
         self.a_shape = (int(A.nrows), int(A.ncols))  # the caller's A (read_A's shape)
 
     def _csr(self, M, keep) -> _Csr:
@@ -383,7 +386,7 @@ class DynamicSpGEMM:
         s = _stream(stream)
         nnz = C.c_int64()
         self._check(fn(self._h, C.byref(nnz), None, None, None, 0, s))
-        n = self.info()["n"] if nrows is None else nrows
+        n = self._n if nrows is None else nrows
         rp = _host_empty(n + 1, np.int64)
         col = _host_empty(nnz.value, np.int32)
         val = _host_empty(nnz.value, _vdtype(self.sr))
@@ -392,7 +395,7 @@ class DynamicSpGEMM:
 
     def read_C(self, stream=None) -> "CsrArrays":
         """C' in canonical CSR (host numpy arrays)."""
-        return self._read(self._lib.dspg_read_C, self.info()["m"], stream)
+        return self._read(self._lib.dspg_read_C, self._m, stream)
 
     def read_bloom(self, stream=None) -> "CsrArrays":
         """C's Bloom filter F (handles built with ``bloom=True``) in canonical
@@ -400,13 +403,13 @@ class DynamicSpGEMM:
         s = _stream(stream)
         nnz = C.c_int64()
         self._check(self._lib.dspg_read_bloom(self._h, C.byref(nnz), None, None, None, 0, s))
-        n = self.info()["n"]
+        n = self._n
         rp = _host_empty(n + 1, np.int64)
         col = _host_empty(nnz.value, np.int32)
         words = _host_empty(nnz.value, np.int64).view(np.uint64)
         self._check(self._lib.dspg_read_bloom(self._h, C.byref(nnz), rp.ctypes.data, col.ctypes.data,
                                               words.ctypes.data, 0, s))
-        return CsrArrays(n, self.info()["m"], rp, col, words)
+        return CsrArrays(n, self._m, rp, col, words)
 
     def read_A(self, stream=None) -> "CsrArrays":
         """A' in canonical CSR (host numpy arrays), in the caller's coordinates."""
@@ -418,7 +421,7 @@ class DynamicSpGEMM:
         nnz = C.c_int64()
         s = _stream(stream)
         self._check(self._lib.dspg_read_C(self._h, C.byref(nnz), None, None, None, 1, s))
-        n = self.info()["n"]
+        n = self._n
         rp = torch.empty(n + 1, dtype=torch.int64, device="cuda")
         col = torch.empty(max(nnz.value, 1), dtype=torch.int32, device="cuda")
         val = torch.empty(max(nnz.value, 1), dtype=torch.float64 if self.sr == PLUS_TIMES_F64 else torch.int32,
@@ -572,7 +575,7 @@ class DynamicSpGEMM:
         import torch
         keep: list = []
         if rows is None:
-            n = self.info()["n"]
+            n = self._n
             rp = None
         else:
             rows = rows if _is_torch(rows) and rows.is_cuda else torch.as_tensor(np.asarray(rows, np.int32)).cuda()

@@ -54,3 +54,53 @@ def test_rows_in_order_at_every_width(dspg, m, sr):
     sabs = Ao.multiply_rows(Bo, pick, absval=True)[2] if sr == PLUS_TIMES_F64 else None
     assert_rows_match(*g.read_rows_C(pick), orp, ocol, oval, sabs, "listed rows")
     g.close()
+
+
+def test_fill_call_takes_the_row_pointers_of_its_count_call_only(dspg):
+    """The fill call of a two-call read of all of C, or of listed rows, uses the
+    row pointers of its count call; a batch, a read of the affected rows or of
+    A in between makes it compute them again."""
+    import ctypes
+    sr = MIN_PLUS_I32
+    rng = np.random.default_rng(3)
+    rows = [rng.choice(300, size=int(rng.integers(0, 9)), replace=False) for _ in range(300)]
+    A = _csr(rows, 300, sr, rng)
+    g = dspg.DynamicSpGEMM(A)
+    Ao = OMat.from_csr(A)
+    lib, h = dspg.load(), g._h
+
+    def batch(seed):
+        from workloads import random_batch
+        b = random_batch(300, 300, 40, seed, sr, A=Ao.to_csr())
+        g.apply_batch(b)
+        Ao.apply(b)
+
+    def count(listed):
+        nnz = ctypes.c_int64()
+        if listed is None:
+            assert lib.dspg_read_C(h, ctypes.byref(nnz), None, None, None, 0, None) == 0
+        else:
+            assert lib.dspg_read_rows_C(h, listed.ctypes.data, len(listed), ctypes.byref(nnz), None, None, None, 0, None) == 0
+        return nnz
+
+    def fill(listed, nnz):
+        n = A.nrows if listed is None else len(listed)
+        rp, col, val = np.zeros(n + 1, np.int64), np.zeros(100000, np.int32), np.zeros(100000, np.int32)
+        out = (rp.ctypes.data, col.ctypes.data, val.ctypes.data, 0, None)
+        if listed is None:
+            assert lib.dspg_read_C(h, ctypes.byref(nnz), *out) == 0
+        else:
+            assert lib.dspg_read_rows_C(h, listed.ctypes.data, len(listed), ctypes.byref(nnz), *out) == 0
+        every = np.arange(A.nrows, dtype=np.int32) if listed is None else listed
+        assert_rows_match(rp, col[: rp[-1]], val[: rp[-1]], *Ao.multiply_rows(Ao, every), what="fill")
+
+    some = rng.permutation(300)[:50].astype(np.int32)
+    batch(1)
+    for listed in (None, some):
+        for between in (lambda: None, lambda: batch(2), lambda: g.read_affected(), lambda: g.read_A(),
+                        lambda: count(some if listed is None else None)):
+            nnz = count(listed)
+            between()
+            fill(listed, nnz)
+            fill(listed, nnz)
+    g.close()
