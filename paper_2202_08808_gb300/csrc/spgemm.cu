@@ -916,8 +916,25 @@ k_num_thread_merge(MatView A, MatView B, MatView C, CJob J, Ctl *ctl, unsigned m
 // the row in column order.  The words are distinct, so the sort needs no
 // tie rule, and it has no data-dependent branches.  Columns must leave room
 // for the slot bits (sort_cols_ok).
+//
+// Bound by shared-memory and shuffle wavefronts (73% of their peak; issue 54%,
+// the double-precision pipe 31%) and the latency of the row's four loads one
+// after the other.  On the square of the 128^3 stencil (2.1 million rows of 49
+// products): 1230 us with a shuffle search per product, 8 conditional
+// additions for the carry, slots of the warp's groups in the same banks and
+// entries stored where the lanes hold them; 1165 with the products' A entries
+// from a mask of the row's starts and one addition, 1126 with the groups'
+// slots padded apart, 1081 with the row stored from the slots in stretches.
+// A values kept per A entry instead of per product measured the same and
+// spilled.
 constexpr int GS_EPL = 8;
 constexpr int GS_NT = 256;
+
+// slots of a group with its pad
+__host__ __device__ constexpr int group_sort_ld(int G) { return G * GS_EPL + (G < 32 ? G : 0); }
+constexpr size_t group_sort_smem(int G, size_t vsize) {
+    return (size_t)(GS_NT / G) * group_sort_ld(G) * (4 + 2 * vsize) + (G == 8 ? GS_NT * (8 + vsize) : 0);
+}
 
 template <int SR, int G>
 __global__ void __launch_bounds__(GS_NT, 4)
@@ -928,17 +945,24 @@ k_num_group_sort(MatView A, MatView B, MatView C, CJob J, Ctl *ctl, unsigned mas
     constexpr int LOGN = G == 8 ? 6 : (G == 16 ? 7 : 8);
     static_assert((1 << LOGN) == N, "words per group");
     constexpr uint32_t PAD = 0xffffffffu;  // empty word: sorts last, never written
-    // the group's N product slots: B column, A value, B value
-    __shared__ int32_t s_col[GS_NT / G * N];
-    __shared__ T s_a[GS_NT / G * N];
-    __shared__ T s_b[GS_NT / G * N];
+    // the groups' product slots (B column, A value, B value: N each and a
+    // pad, so that the groups of a warp, which fill and read the same slots
+    // together, lie in different banks) and, for G == 8, the chunk's A
+    // entries with a B row, in order: the B entry of product p is rel + p,
+    // its A value ea
+    extern __shared__ __align__(16) unsigned char smem[];
+    constexpr int LD = group_sort_ld(G);
+    T *s_a = (T *)smem, *s_b = s_a + GS_NT / G * LD;
+    int64_t *s_rel = (int64_t *)(s_b + GS_NT / G * LD);
+    T *s_ea = (T *)(s_rel + (G == 8 ? GS_NT : 0));
+    int32_t *s_col = (int32_t *)(s_ea + (G == 8 ? GS_NT : 0));
     if (__any_sync(0xffffffffu, failed(ctl, mask))) return;  // a warp leaves as a whole
     const int lane = threadIdx.x & 31;
     const int gl = lane & (G - 1), gw = lane / G;
     const unsigned gmask = G == 32 ? 0xffffffffu : (((1u << G) - 1u) << (gw * G));
-    int32_t *scol = s_col + (threadIdx.x / G) * N;
-    T *sa = s_a + (threadIdx.x / G) * N;
-    T *sb = s_b + (threadIdx.x / G) * N;
+    int32_t *scol = s_col + (threadIdx.x / G) * LD;
+    T *sa = s_a + (threadIdx.x / G) * LD;
+    T *sb = s_b + (threadIdx.x / G) * LD;
     const long long ngroups = ((long long)gridDim.x * GS_NT) / G;
     const T *Av = (const T *)A.val;
     const T *Bv = (const T *)B.val;
@@ -975,6 +999,45 @@ k_num_group_sort(MatView A, MatView B, MatView C, CJob J, Ctl *ctl, unsigned mas
             if (base + total > N) {  // the bin's bound rules this out; guard the slots anyway
                 over = true;
                 break;
+            }
+            if constexpr (G == 8) {
+                // products by position: bit p of the group's mask is set
+                // where a B row starts, so product p belongs to the A entry
+                // whose rank is the number of bits up to p
+                int64_t *rel = s_rel + threadIdx.x / G * G;
+                T *ea = s_ea + threadIdx.x / G * G;
+                const int excl = incl - blen;
+                const unsigned some = __ballot_sync(gmask, blen > 0) >> (gw * G);
+                uint32_t lo = blen > 0 && excl < 32 ? 1u << excl : 0u;
+                uint32_t hi = blen > 0 && excl >= 32 ? 1u << (excl - 32) : 0u;
+                if (blen > 0) {
+                    const int rank = __popc(some & ((1u << gl) - 1u));
+                    rel[rank] = boff - excl;
+                    ea[rank] = av;
+                }
+#pragma unroll
+                for (int d = 1; d < G; d <<= 1) {
+                    lo |= __shfl_xor_sync(gmask, lo, d, G);
+                    hi |= __shfl_xor_sync(gmask, hi, d, G);
+                }
+                __syncwarp(gmask);
+                const int nlo = __popc(lo);
+#pragma unroll
+                for (int e = 0; e < GS_EPL; e++) {
+                    const int slot = e * G + gl, p = slot - base;
+                    if (p >= 0 && p < total) {
+                        const uint32_t up_to = 0xffffffffu >> (31 - (p & 31));  // bits 0 .. p mod 32
+                        const int s = (p < 32 ? __popc(lo & up_to) : nlo + __popc(hi & up_to)) - 1;
+                        const int64_t q = rel[s] + p;
+                        cp_async_4(&scol[slot], B.col + q);
+                        if (sizeof(T) == 8) cp_async_8(&sb[slot], Bv + q);
+                        else cp_async_4(&sb[slot], Bv + q);
+                        sa[slot] = ea[s];
+                    }
+                }
+                __syncwarp(gmask);  // rel and ea are read before the next chunk or row writes them
+                base += total;
+                continue;
             }
 #pragma unroll
             for (int e = 0; e < GS_EPL; e++) {
@@ -1092,11 +1155,17 @@ k_num_group_sort(MatView A, MatView B, MatView C, CJob J, Ctl *ctl, unsigned mas
         // the carry of a linked lane joins its first run, whose last word is
         // the only one of that run an output can come from
         const T carry = __shfl_up_sync(gmask, run, 1, G);
-        if (link)
+        // one addition at the word that ends the run, found by selects (an
+        // addition per word under a condition took the double-precision
+        // pipe, 16 cycles a warp, eight times)
+        T ends = v[0];
 #pragma unroll
-            for (int e = 0; e < GS_EPL; e++)
-                if (col[e] == first && (e + 1 == GS_EPL || col[e + 1 < GS_EPL ? e + 1 : e] != first))
-                    v[e] = Sr<SR>::add(carry, v[e]);
+        for (int e = 1; e < GS_EPL; e++)
+            if (col[e] == first) ends = v[e];
+        ends = Sr<SR>::add(carry, ends);
+#pragma unroll
+        for (int e = 0; e < GS_EPL; e++)
+            if (link && col[e] == first && (e + 1 == GS_EPL || col[e + 1 < GS_EPL ? e + 1 : e] != first)) v[e] = ends;
         // the last word of each run holds the entry; its rank among the
         // row's runs is its place in the output
         const int32_t next_first = __shfl_down_sync(gmask, first, 1, G);
@@ -1118,14 +1187,21 @@ k_num_group_sort(MatView A, MatView B, MatView C, CJob J, Ctl *ctl, unsigned mas
         if (gl == 0) dest = c_row_dest(C, J, ctl, i, n);
         dest = __shfl_sync(gmask, dest, 0, G);
         if (dest >= 0) {
+            // through the slots, so that the row is stored in whole stretches
+            __syncwarp(gmask);  // every lane has read the slots
 #pragma unroll
             for (int e = 0; e < GS_EPL; e++) {
                 const int32_t nk = e + 1 < GS_EPL ? col[e + 1] : (gl + 1 < G ? next_first : -1);
                 if (col[e] >= 0 && nk != col[e]) {
-                    C.col[dest + w] = col[e];
-                    Cv[dest + w] = v[e];
+                    scol[w] = col[e];
+                    sb[w] = v[e];
                     w++;
                 }
+            }
+            __syncwarp(gmask);
+            for (int q = gl; q < n; q += G) {
+                C.col[dest + q] = scol[q];
+                Cv[dest + q] = sb[q];
             }
             if (gl == 0) C.len[i] = n;
         }
@@ -2087,8 +2163,9 @@ static void launch_group_hash(const MatView &A, const MatView &B, const MatView 
 template <int SR, int G>
 static void launch_group_sort(const MatView &A, const MatView &B, const MatView &C, const CJob &J, Ctl *ctl,
                               unsigned mask, int bin, cudaStream_t s, int num_sms) {
-    static const int per_sm = resident_per_sm(k_num_group_sort<SR, G>, GS_NT, 0);
-    launch_k(k_num_group_sort<SR, G>, grid_for(num_sms * per_sm, J.rows_hint, GS_NT / G), GS_NT, 0, s, A, B, C, J,
+    constexpr size_t smem = group_sort_smem(G, sizeof(typename Sr<SR>::T));
+    static const int per_sm = resident_per_sm(k_num_group_sort<SR, G>, GS_NT, smem);
+    launch_k(k_num_group_sort<SR, G>, grid_for(num_sms * per_sm, J.rows_hint, GS_NT / G), GS_NT, smem, s, A, B, C, J,
              ctl, mask, bin);
 }
 
