@@ -419,6 +419,8 @@ struct dspg_handle {
     Ctl *ctl = nullptr;   // device
     Ctl *hctl = nullptr;      // pinned, mapped host mirror
     Ctl *hctl_dev = nullptr;  // its device address
+    ReadOut *hro = nullptr;      // behind hctl: what a read found
+    ReadOut *hro_dev = nullptr;  // its device address
     UpdWs wA, wB, wAT;
     CWs wc;
     // grow-only scratch of the read calls (row list, lengths, row pointers,
@@ -1400,8 +1402,12 @@ void fill_rows_out(dspg_handle *h, DevMat &M, const MatView &V, int vs, const in
     h->rd.res.reserve(1);
     CK(cudaMemsetAsync(h->rd.res.p, 0, sizeof(ReadOut), s));
     auto rows_out = [&](int32_t *oc, void *ov) {
-        read_rows_out(rows, n, nullptr, V, vs, rp, nullptr, nnz, oc, ov, nullptr, nullptr, longs, huge, h->rd.res.p, s,
-                      h->num_sms);
+        read_rows_out(rows, n, nullptr, V, vs, rp, nullptr, nnz, oc, ov, nullptr, nullptr, longs, huge, h->rd.res.p,
+                      nullptr, s, h->num_sms);
+        if (!read_has_huge(V.ncols)) {
+            if (on_device) CK(cudaStreamSynchronize(s));
+            return;
+        }
         ReadOut ro{};
         CK(cudaMemcpyAsync(&ro, h->rd.res.p, sizeof(ReadOut), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
@@ -2335,8 +2341,10 @@ dspg_status dspg_build_form(dspg_handle **out, const dspg_csr *A, const dspg_csr
         for (cudaEvent_t *e : {&h->evIn, &h->evFork, &h->evDetect, &h->evSide, &h->evSize})
             CK(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
         if (const char *env = getenv("DSPG_NO_GRAPHS")) h->use_graphs = env[0] == '0';
-        CK(cudaHostAlloc((void **)&h->hctl, sizeof(Ctl), cudaHostAllocMapped));
+        CK(cudaHostAlloc((void **)&h->hctl, sizeof(Ctl) + sizeof(ReadOut), cudaHostAllocMapped));
         CK(cudaHostGetDevicePointer((void **)&h->hctl_dev, h->hctl, 0));
+        h->hro = (ReadOut *)(h->hctl + 1);
+        h->hro_dev = (ReadOut *)(h->hctl_dev + 1);
         CK(cudaMalloc((void **)&h->d_args, 3 * sizeof(InArgs)));
         CK(cudaHostAlloc((void **)&h->h_args, 3 * sizeof(InArgs), cudaHostAllocMapped));
         CK(cudaHostGetDevicePointer((void **)&h->h_args_dev, h->h_args, 0));
@@ -2624,13 +2632,17 @@ dspg_status dspg_read_affected_C(dspg_handle *h, int64_t rows_cap, int64_t nnz_c
             w.huge_l.reserve(std::max<int64_t>(n, 1));
             w.c.reserve(std::max<int64_t>(nnz_cap, 1));
             w.v.reserve(std::max<int64_t>(nnz_cap, 1) * std::max(h->vsize, 1));
+            h->hro->flags = READ_UNORDERED;  // until the read says otherwise
             read_rows_out(w.r.p, n, nullptr, h->C.view(), h->vsize, rp, w.chunk_ex.p + nch, nnz_cap, w.c.p,
-                          (void *)w.v.p, dcol, dval, w.long_l.p, w.huge_l.p, w.res.p, s, h->num_sms);
-            ReadOut ro{};
-            CK(cudaMemcpyAsync(&ro, w.res.p, sizeof(ReadOut), cudaMemcpyDeviceToHost, s));
+                          (void *)w.v.p, dcol, dval, w.long_l.p, w.huge_l.p, w.res.p, h->hro_dev, s, h->num_sms);
+            unsigned n_huge = 0;
+            if (read_has_huge(h->C.ncols))
+                CK(cudaMemcpyAsync(&n_huge, &w.res.p->n_huge, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
             if (n > 0 && !drows) CK(cudaMemcpyAsync(rows, w.r.p, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, s));
             if (!drp) CK(cudaMemcpyAsync(rowptr, rp, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToHost, s));
             CK(cudaStreamSynchronize(s));
+            ReadOut ro = *h->hro;
+            ro.n_huge = n_huge;
             if (!(ro.flags & READ_UNORDERED)) {
                 *nrows_out = n;
                 *nnz_out = ro.nnz;
@@ -2724,15 +2736,21 @@ dspg_status dspg_apply_read_affected(dspg_handle *h, const dspg_updates *dA, con
             ReadOut ro{};
             try {
                 run_first(h, s, false);
+                h->hro->flags = READ_UNORDERED;  // until the read says otherwise
                 // behind the batch: R's size from the device, bounded by cap
                 const long long *n_dev = &h->ctl->n_affected;
                 read_order_rowptr(h->wc.R.p, h->wc.rchunk.p, nch, rc, n_dev, cap, &h->ctl->status, h->C.len.p, w.r.p,
                                   w.lens.p, w.chunk_cnt.p, w.chunk_ex.p + nch, w.rp.p, drows, drp, w.res.p, s,
                                   h->num_sms);
                 read_rows_out(w.r.p, rc, n_dev, h->C.view(), h->vsize, w.rp.p, w.chunk_ex.p + nch, nnz_cap, w.c.p,
-                              (void *)w.v.p, dcol, dval, w.long_l.p, w.huge_l.p, w.res.p, s, h->num_sms);
-                CK(cudaMemcpyAsync(&ro, w.res.p, sizeof(ReadOut), cudaMemcpyDeviceToHost, s));
+                              (void *)w.v.p, dcol, dval, w.long_l.p, w.huge_l.p, w.res.p, h->hro_dev, s,
+                              h->num_sms);
+                unsigned n_huge = 0;
+                if (read_has_huge(h->C.ncols))
+                    CK(cudaMemcpyAsync(&n_huge, &w.res.p->n_huge, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
                 CK(cudaStreamSynchronize(s));
+                ro = *h->hro;
+                ro.n_huge = n_huge;
                 // a batch that needs a second pass changes C after the read
                 clean = h->hctl->status == 0 && h->hctl->n_ovf <= 0;
                 if (h->prof) stage_times_from_events(h);

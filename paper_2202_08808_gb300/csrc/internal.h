@@ -310,12 +310,15 @@ enum : unsigned { READ_TOO_SMALL = 1u, READ_UNORDERED = 2u };
 // as the scratch of the longer rows.  The values' array may be null: then
 // columns only.  Lists: one entry per row of more than 64 entries
 // (long_list), and in a C of more than 2^22 columns per row of more than
-// 16384 (huge_list); res zeroed by the caller.
+// 16384 (huge_list); res zeroed by the caller.  host_res (or null): mapped
+// host memory that gets what the host needs of res, all but n_huge.
 // n_dev (or null): n read on the device, n then bounding it (grid sizes).
 void read_rows_out(const int32_t *rows, int64_t n, const long long *n_dev, const MatView &M, int vsize,
                    const int64_t *rp, const int64_t *r_total, int64_t nnz_cap, int32_t *dst_col, void *dst_val,
                    int32_t *out_col, void *out_val, int64_t *long_list, int64_t *huge_list, ReadOut *res,
-                   cudaStream_t s, int num_sms);
+                   ReadOut *host_res, cudaStream_t s, int num_sms);
+// Whether a read of a C of that many columns may leave rows to the huge list.
+bool read_has_huge(int64_t ncols);
 // R (n rows, as collected: ascending within each 8192-row chunk, chunk c's
 // rows at chunk[2c] with chunk[2c+1] of them) into out in row order; cnt and
 // ex (nch + 1) and tmp (scan_tmp_entries(nch) + 1) are scratch, and ex[nch]

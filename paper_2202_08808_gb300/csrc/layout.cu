@@ -265,10 +265,82 @@ k_read_rowptr(const long long *chunk, int nch, int64_t n_arg, const long long *n
     }
 }
 
+// The same for at most RS_MAX rows, in one launch of one block: a thread
+// takes four consecutive places of R, finds their chunk by a search of the
+// scanned counts in shared memory, and the four loads of each step are in
+// flight together.  Two launches of many blocks take 9 us on a few thousand
+// rows, most of it their own latency; this one 6.
+constexpr int64_t RS_MAX = 4 * RD_NT;
+
+__global__ void __launch_bounds__(RD_NT)
+k_read_small(const int32_t *R, const long long *chunk, int nch, int64_t n_arg, const long long *n_dev, int64_t rows_cap,
+             const unsigned *status, const int32_t *len, int32_t *out, int64_t *r_total, int64_t *rp, int32_t *h_rows,
+             int64_t *h_rp, ReadOut *res) {
+    pdl_begin();
+    __shared__ int64_t s_ex[RD_NT * RD_IPT], s_b[RD_NT * RD_IPT];
+    __shared__ int64_t s_w[33];
+    const int tid = threadIdx.x;
+    const int64_t n = n_dev ? (int64_t)*n_dev : n_arg;
+    const bool skip = (status && *status) || n < 0 || n > rows_cap || n > RS_MAX;
+    for (int c = tid; c < nch; c += RD_NT) s_b[c] = chunk[2 * c];
+    const int64_t tot = rd_scan_table([&](int c) { return (int64_t)chunk[2 * c + 1]; }, nch, s_ex, s_w);
+    if (tid == 0) {
+        *r_total = skip ? -1 : tot;
+        if (res) {
+            ReadOut z{};
+            z.nr = n;
+            *res = z;
+        }
+    }
+    if (skip || tot != n) return;
+    int32_t r[4];
+    int64_t L[4], sum = 0;
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        const int64_t t = (int64_t)tid * 4 + j;
+        r[j] = 0;
+        if (t < n) {
+            const int c = (int)upper_bound_dev<int64_t>(s_ex, 0, nch, t) - 1;  // the last chunk that starts at or before t
+            const int64_t b = s_b[c] + t - s_ex[c];
+            r[j] = R[b >= 0 && b < n ? b : 0];
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        const int64_t t = (int64_t)tid * 4 + j;
+        L[j] = t < n ? len[r[j]] : 0;
+        sum += L[j];
+        if (t < n) {
+            out[t] = r[j];
+            if (h_rows) h_rows[t] = r[j];
+        }
+    }
+    int64_t nnz = 0;
+    int64_t e = rd_block_scan(sum, s_w, &nnz);
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        const int64_t t = (int64_t)tid * 4 + j;
+        if (t < n) {
+            rp[t] = e;
+            if (h_rp) h_rp[t] = e;
+        }
+        e += L[j];
+    }
+    if (tid == 0) {
+        rp[n] = nnz;
+        if (h_rp) h_rp[n] = nnz;
+    }
+}
+
 void read_order_rowptr(const int32_t *R, const long long *chunk, int64_t nch, int64_t n, const long long *n_dev,
                        int64_t rows_cap, const unsigned *status, const int32_t *len, int32_t *out, int32_t *lens,
                        int64_t *S, int64_t *r_total, int64_t *rp, int32_t *h_rows, int64_t *h_rp, ReadOut *res,
                        cudaStream_t s, int num_sms) {
+    if (n <= RS_MAX) {
+        launch_k(k_read_small, 1, RD_NT, 0, s, R, chunk, (int)nch, n, n_dev, rows_cap, status, len, out, r_total, rp,
+                 h_rows, h_rp, res);
+        return;
+    }
     const unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nch, (int64_t)num_sms * 2));
     launch_k(k_read_order, g, RD_NT, 0, s, R, chunk, (int)nch, n, n_dev, rows_cap, status, len, out, lens, S, r_total,
              h_rows, res);
@@ -364,7 +436,8 @@ constexpr int RS_PW = RS_ROWS / (RS_NT / 32);  // rows of a warp
 template <typename T>
 __global__ void __launch_bounds__(RS_NT)
 k_read_short(const int32_t *rows, int64_t n_arg, const long long *n_dev, MatView M, const int64_t *rp,
-             const int64_t *r_total, int64_t nnz_cap, int32_t *out_col, T *out_val, int64_t *long_list, ReadOut *res) {
+             const int64_t *r_total, int64_t nnz_cap, int32_t *out_col, T *out_val, int64_t *long_list, ReadOut *res,
+             ReadOut *host_res) {
     pdl_begin();
     __shared__ T s_val[RS_ROWS * SORT_SHORT];
     __shared__ int32_t s_col[RS_ROWS * SORT_SHORT];
@@ -376,6 +449,13 @@ k_read_short(const int32_t *rows, int64_t n_arg, const long long *n_dev, MatView
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         res->nnz = nnz;
         if (bad) atomicOr(&res->flags, bad);
+        if (host_res) {  // all that the host needs, but for a very wide C's longest rows
+            ReadOut z{};
+            z.nnz = nnz;
+            z.flags = bad;
+            z.nr = n;
+            *host_res = z;
+        }
     }
     if (bad) return;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -702,11 +782,11 @@ template <typename T>
 static void read_rows_out_t(const int32_t *rows, int64_t n, const long long *n_dev, const MatView &M, bool has_val,
                             const int64_t *rp, const int64_t *r_total, int64_t nnz_cap, int32_t *dst_col, T *dst_val,
                             int32_t *out_col, T *out_val, int64_t *long_list, int64_t *huge_list, ReadOut *res,
-                            cudaStream_t s, int num_sms) {
+                            ReadOut *host_res, cudaStream_t s, int num_sms) {
     // n on the device: n is the host's bound on it, which sizes the grids
     launch_k(k_read_short<T>, blocks_for(std::max<int64_t>(n, 1), RS_ROWS, (int64_t)num_sms * 8), RS_NT, 0, s, rows, n,
              n_dev, M, rp, r_total, nnz_cap, out_col ? out_col : dst_col,
-             has_val ? (out_col ? out_val : dst_val) : (T *)nullptr, long_list, res);
+             has_val ? (out_col ? out_val : dst_val) : (T *)nullptr, long_list, res, host_res);
     if (M.ncols <= OL_MAX_COLS) {
         const int W = (int)std::min<int64_t>(OL_W, std::max<int64_t>(1, (M.ncols + 1023) / 1024) * 1024);
         const size_t smem = order_long_smem(W);
@@ -729,17 +809,19 @@ static void read_rows_out_t(const int32_t *rows, int64_t n, const long long *n_d
              rows, M, rp, (const int64_t *)long_list, dst_col, dst_val, out_col, out_val, has_val, huge_list, res);
 }
 
+bool read_has_huge(int64_t ncols) { return ncols > OL_MAX_COLS; }
+
 void read_rows_out(const int32_t *rows, int64_t n, const long long *n_dev, const MatView &M, int vsize,
                    const int64_t *rp, const int64_t *r_total, int64_t nnz_cap, int32_t *dst_col, void *dst_val,
                    int32_t *out_col, void *out_val, int64_t *long_list, int64_t *huge_list, ReadOut *res,
-                   cudaStream_t s, int num_sms) {
+                   ReadOut *host_res, cudaStream_t s, int num_sms) {
     const bool has_val = vsize && M.val && (out_col ? out_val != nullptr : dst_val != nullptr);
     if (vsize == 8)
         read_rows_out_t<double>(rows, n, n_dev, M, has_val, rp, r_total, nnz_cap, dst_col, (double *)dst_val, out_col,
-                                (double *)out_val, long_list, huge_list, res, s, num_sms);
+                                (double *)out_val, long_list, huge_list, res, host_res, s, num_sms);
     else
         read_rows_out_t<int32_t>(rows, n, n_dev, M, has_val, rp, r_total, nnz_cap, dst_col, (int32_t *)dst_val, out_col,
-                                 (int32_t *)out_val, long_list, huge_list, res, s, num_sms);
+                                 (int32_t *)out_val, long_list, huge_list, res, host_res, s, num_sms);
 }
 
 // Rows too long for a CTA's shared memory, sorted all at once: the packed

@@ -104,3 +104,35 @@ def test_fill_call_takes_the_row_pointers_of_its_count_call_only(dspg):
             fill(listed, nnz)
             fill(listed, nnz)
     g.close()
+
+
+@pytest.mark.parametrize("nr", [1, 3, 1023, 1025, 4095, 4096, 4097, 9000])
+def test_affected_rows_around_the_one_block_read(dspg, nr):
+    """R and its row pointers come from one block up to 4096 rows and from many
+    beyond: both one-call reads, with R spread over the bitmap's chunks."""
+    import torch
+    from workloads import OP_SET, Batch
+    rng = np.random.default_rng(nr)
+    n, k, m = 30000, 150, 40
+    A = _csr([rng.choice(k, size=int(rng.integers(0, 4)), replace=False) for _ in range(n)], k, MIN_PLUS_I32, rng)
+    B = _csr([rng.choice(m, size=int(rng.integers(0, 6)), replace=False) for _ in range(k)], m, MIN_PLUS_I32, rng)
+    g, g2 = dspg.DynamicSpGEMM(A, B), dspg.DynamicSpGEMM(A, B)
+    Ao, Bo = OMat.from_csr(A), OMat.from_csr(B)
+    for room in (nr, nr + 300):  # the arrays' room bounds what the launch is sized for
+        rows = np.sort(rng.choice(n, size=nr, replace=False)).astype(np.int32)
+        b = Batch(rng.permutation(rows), rng.integers(0, k, nr).astype(np.int32), rng.integers(1, 99, nr).astype(np.int32),
+                  np.full(nr, OP_SET, np.uint8))
+        out = (torch.empty(room, dtype=torch.int32, pin_memory=True).numpy(),
+               torch.empty(room + 1, dtype=torch.int64, pin_memory=True).numpy(),
+               torch.empty(room * 40 + 1, dtype=torch.int32, pin_memory=True).numpy(),
+               torch.empty(room * 40 + 1, dtype=torch.int32, pin_memory=True).numpy())
+        _, one = g.apply_read_affected(b, out=out)
+        g2.apply_batch(b)
+        two = g2.read_affected()
+        Ao.apply(b)
+        want = Ao.multiply_rows(Bo, rows)
+        for got in (one, two):
+            assert np.array_equal(got[0], rows)
+            assert_rows_match(*got[1:], *want, what=f"{nr} rows")
+    g.close()
+    g2.close()
