@@ -1117,6 +1117,14 @@ void reset_c_counters(dspg_handle *h, cudaStream_t s) {
     reset_range(h, from, sizeof(Ctl) - (size_t)(from - (char *)c), s);
 }
 
+void *device_view(void *p);
+
+// Entries of a page-locked batch that is read in place: those of the one-launch
+// sorts, which read every entry once and its value and operation once more
+// where it goes.  A batch and read of 16 updates takes 94.5 us so against 98.8
+// with the four copies, of 10^4 266 against 271.
+constexpr int64_t kInPlace = 16384;
+
 // Host batches are copied to the device; device batches are read where
 // they are.  Either way the pointers go to the argument block slot k.
 // A transposed operand takes the caller's (i, j) as (j, i): the row and
@@ -1127,11 +1135,26 @@ void upload(dspg_handle *h, UpdWs &w, const dspg_updates *u, BatchIn &in, int k,
     h->h_args[k] = InArgs{nullptr, nullptr, nullptr, nullptr, 0};
     if (in.n <= 0) return;
     const int32_t *ur = swap ? u->col : u->row, *uc = swap ? u->row : u->col;
+    // a short batch in page-locked memory is read in place too, over the C2C
+    // link, by the sort (its one reader), if its arrays are aligned for loads
+    const void *dr = nullptr, *dc = nullptr, *dv = nullptr, *dp = nullptr;
+    const bool aligned = ((uintptr_t)ur | (uintptr_t)uc) % sizeof(int32_t) == 0 && (uintptr_t)u->val % h->vsize == 0;
+    if (!u->on_device && in.n <= kInPlace && aligned) {
+        dr = device_view(const_cast<int32_t *>(ur));
+        dc = dr ? device_view(const_cast<int32_t *>(uc)) : nullptr;
+        dv = dc ? device_view(const_cast<void *>(u->val)) : nullptr;
+        dp = dv ? device_view(const_cast<uint8_t *>(u->op)) : nullptr;
+    }
     if (u->on_device) {
         in.row = ur;
         in.col = uc;
         in.val = u->val;
         in.op = u->op;
+    } else if (dp) {
+        in.row = (const int32_t *)dr;
+        in.col = (const int32_t *)dc;
+        in.val = dv;
+        in.op = (const uint8_t *)dp;
     } else {
         CK(cudaMemcpyAsync(w.in_row.p, ur, sizeof(int32_t) * in.n, cudaMemcpyHostToDevice, s));
         CK(cudaMemcpyAsync(w.in_col.p, uc, sizeof(int32_t) * in.n, cudaMemcpyHostToDevice, s));
