@@ -292,6 +292,19 @@ struct SortScratch {  // for `total` entries: keys, indices (two each), radix co
 void sort_listed_rows(const int64_t *rowptr, const int64_t *listed, const int64_t *pre, int nl, int64_t total,
                       int cb, int32_t *col, void *val, int vsize, const SortScratch &w, cudaStream_t s, int num_sms);
 void lens_of_rows(const int32_t *rows, int64_t n, const int32_t *len, int32_t *out, cudaStream_t s);
+#ifdef __CUDACC__
+// Blocks of kern of nt threads (and no dynamic shared memory) that an SM holds.
+template <typename K>
+inline int resident_blocks(K kern, int nt) {
+    int nb = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, nt, 0) != cudaSuccess || nb < 1) {
+        cudaGetLastError();  // the launch itself reports a kernel that cannot run
+        nb = 1;
+    }
+    return nb;
+}
+#endif
+
 // What a read of rows found (layout.cu), for the host synchronisation after it.
 struct ReadOut {
     long long nnz;   // entries of the rows (rp[n])

@@ -783,8 +783,12 @@ static void read_rows_out_t(const int32_t *rows, int64_t n, const long long *n_d
                             const int64_t *rp, const int64_t *r_total, int64_t nnz_cap, int32_t *dst_col, T *dst_val,
                             int32_t *out_col, T *out_val, int64_t *long_list, int64_t *huge_list, ReadOut *res,
                             ReadOut *host_res, cudaStream_t s, int num_sms) {
-    // n on the device: n is the host's bound on it, which sizes the grids
-    launch_k(k_read_short<T>, blocks_for(std::max<int64_t>(n, 1), RS_ROWS, (int64_t)num_sms * 8), RS_NT, 0, s, rows, n,
+    // n on the device: n is the host's bound on it, which sizes the grids.
+    // One wave of resident blocks: a partial second one left SMs idle (the
+    // 128^3 stencil's square into device memory: 398 us with 8 blocks an SM
+    // launched of which 5 fit, 354 so).
+    static const int per_sm = resident_blocks(k_read_short<T>, RS_NT);
+    launch_k(k_read_short<T>, blocks_for(std::max<int64_t>(n, 1), RS_ROWS, (int64_t)num_sms * per_sm), RS_NT, 0, s, rows, n,
              n_dev, M, rp, r_total, nnz_cap, out_col ? out_col : dst_col,
              has_val ? (out_col ? out_val : dst_val) : (T *)nullptr, long_list, res, host_res);
     if (M.ncols <= OL_MAX_COLS) {

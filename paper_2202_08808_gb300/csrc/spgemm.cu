@@ -1858,7 +1858,8 @@ void run_size_bins(const MatView &A, const MatView &B, const MatView &C, const C
                    unsigned mask, cudaStream_t s, int num_sms) {
     if (max_rows <= 0) return;
     int64_t g = (max_rows + 255) / 256;
-    if (g > num_sms * 8) g = num_sms * 8;
+    static const int per_sm = resident_blocks(k_size_bins, 256);  // one wave, as a block's rounds are dealt out evenly (105 to 87 us on 2.1 million rows)
+    if (g > (int64_t)num_sms * per_sm) g = (int64_t)num_sms * per_sm;
     if (g < 1) g = 1;
     launch_k(k_size_bins, (unsigned)g, 256, 0, s, A, B, C, J, ctl, mask);
     if (J.sizing == SIZE_LEARNED) {
