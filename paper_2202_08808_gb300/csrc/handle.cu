@@ -673,6 +673,12 @@ int64_t mat_rowptr(dspg_handle *h, DevMat &M, const int32_t *rows, int64_t n, in
         int32_t *lens = read_scratch(h->rd.lens, lens_l, n);
         lens_of_rows(rows, n, M.len.p, lens, s);
         lp = lens;
+    } else if (h->pending && n > 0) {
+        // the scan reads the lengths twice: while a batch rewrites some of
+        // them, a copy keeps every other row's place right
+        int32_t *lens = read_scratch(h->rd.lens, lens_l, n);
+        CK(cudaMemcpyAsync(lens, M.len.p, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
+        lp = lens;
     }
     int64_t *tmp = read_scratch(h->rd.scan, tmp_l, scan_tmp_entries(n) + 1);
     scan_i32_to_i64(lp, rowptr, n, tmp, s);

@@ -420,6 +420,15 @@ constexpr int RS_NT = 256;         // threads of a k_read_short block
 constexpr int RS_ROWS = 32;        // rows of its tile
 constexpr int RS_PW = RS_ROWS / (RS_NT / 32);  // rows of a warp
 
+// A read may run while an asynchronous batch rewrites other rows of C, and a
+// read of all of C then meets rows that change under it: their entries come
+// out undefined, but every access stays inside the arena and the row's
+// stretch of the result, whose lengths (rp) were taken before.
+__device__ __forceinline__ int64_t row_start(const MatView &M, int64_t r, int64_t len) {
+    const int64_t so = M.off[r], most = M.arena_cap - len;
+    return so <= most ? so : (most > 0 ? most : 0);
+}
+
 // A tile of RS_ROWS consecutive rows per block and round: each warp loads
 // its four rows together, ranks the columns of those out of order by
 // shuffles, and puts the entries at their places in shared memory; the
@@ -470,7 +479,7 @@ k_read_short(const int32_t *rows, int64_t n_arg, const long long *n_dev, MatView
         if (lane < RS_PW && hx < x1) {
             h_d = rp[hx];
             h_len = rp[hx + 1] - h_d;
-            h_so = M.off[rows ? (int64_t)rows[hx] : hx];
+            h_so = row_start(M, rows ? (int64_t)rows[hx] : hx, h_len);
         }
         const bool lng = h_len > SORT_SHORT;
         const unsigned lm = __ballot_sync(0xffffffffu, lng);
@@ -606,7 +615,7 @@ k_order_long(const int32_t *rows, MatView M, const int64_t *rp, const int64_t *l
         const int64_t x = long_list[t];
         const int64_t lo = rp[x];
         const int64_t len = rp[x + 1] - lo;
-        const int64_t so = M.off[rows ? (int64_t)rows[x] : x];
+        const int64_t so = row_start(M, rows ? (int64_t)rows[x] : x, len);
         const int32_t *mc = M.col + so;
         int unsorted = 0;
         int mn = INT32_MAX, mx = -1;
@@ -644,7 +653,7 @@ k_order_long(const int32_t *rows, MatView M, const int64_t *rp, const int64_t *l
 #pragma unroll 4
             for (int64_t e = tid; e < len; e += OL_NT) {
                 const uint32_t c = (uint32_t)(mc[e] - wb);
-                if (c < (uint32_t)W) {
+                if (c < (uint32_t)nb << 10) {
                     atomicOr(&bm[c >> 5], 1u << (c & 31));
                     atomicAdd(&cnt[c >> 10], 1u);
                 }
@@ -674,10 +683,12 @@ k_order_long(const int32_t *rows, MatView M, const int64_t *rp, const int64_t *l
             for (int64_t e = tid; e < len; e += OL_NT) {
                 const int32_t col = mc[e];
                 const uint32_t c = (uint32_t)(col - wb);
-                if (c < (uint32_t)W) {
-                    const int64_t o = lo + first[c >> 10] + pre[c >> 5] + __popc(bm[c >> 5] & ((1u << (c & 31)) - 1u));
-                    dst_col[o] = col;
-                    if (has_val) dst_val[o] = mv[so + e];
+                if (c < (uint32_t)nb << 10) {
+                    const uint32_t o = first[c >> 10] + pre[c >> 5] + __popc(bm[c >> 5] & ((1u << (c & 31)) - 1u));
+                    if (o < (uint64_t)len) {  // always, for a row that does not change meanwhile
+                        dst_col[lo + o] = col;
+                        if (has_val) dst_val[lo + o] = mv[so + e];
+                    }
                 }
             }
             __syncthreads();
@@ -748,7 +759,7 @@ k_sort_long(const int32_t *rows, MatView M, const int64_t *rp, const int64_t *lo
         const int64_t x = long_list[j];
         const int64_t lo = rp[x];
         const int64_t len = rp[x + 1] - lo;
-        const int64_t so = M.off[rows ? (int64_t)rows[x] : x];
+        const int64_t so = row_start(M, rows ? (int64_t)rows[x] : x, len);
         int unsorted = 0;
         for (int64_t e = tid; e + 1 < len; e += nt) unsorted |= M.col[so + e] > M.col[so + e + 1];
         const bool sort = __syncthreads_or(unsorted);

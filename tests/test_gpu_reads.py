@@ -136,3 +136,35 @@ def test_affected_rows_around_the_one_block_read(dspg, nr):
             assert_rows_match(*got[1:], *want, what=f"{nr} rows")
     g.close()
     g2.close()
+
+
+def test_whole_read_while_an_asynchronous_batch_rewrites_rows(dspg):
+    """A read of all of C while a batch runs: the rows the batch cannot change
+    come out whole, whatever the others hold, and the next read is right."""
+    import torch
+    from workloads import random_batch
+    sr = MIN_PLUS_I32
+    rng = np.random.default_rng(12)
+    n, m = 1500, 300000
+    A = _csr([rng.choice(n, size=int(rng.integers(0, 30)), replace=False) for _ in range(n)], n, sr, rng)
+    B = _csr([rng.choice(m, size=int(rng.integers(0, 200)), replace=False) for _ in range(n)], m, sr, rng)
+    g = dspg.DynamicSpGEMM(A, B)
+    Ao, Bo = OMat.from_csr(A), OMat.from_csr(B)
+    every = np.arange(n, dtype=np.int32)
+    side = torch.cuda.Stream()
+    for t in range(6):
+        b = random_batch(n, n, 400, 20 + t, sr, A=Ao.to_csr())
+        g.apply_batch_async(b)
+        mid = g.read_C(stream=side)
+        g.apply_batch_wait()
+        changed = np.zeros(n, bool)
+        changed[g.last_affected()] = True
+        orp, ocol, oval = Ao.multiply_rows(Bo, every)  # before the batch
+        for i in np.nonzero(~changed)[0]:
+            lo, hi = mid.rowptr[i], mid.rowptr[i + 1]
+            assert np.array_equal(mid.col[lo:hi], ocol[orp[i]:orp[i + 1]]), f"batch {t}: row {i}"
+            assert np.array_equal(mid.val[lo:hi], oval[orp[i]:orp[i + 1]]), f"batch {t}: row {i}"
+        Ao.apply(b)
+        C = g.read_C()
+        assert_rows_match(C.rowptr, C.col, C.val, *Ao.multiply_rows(Bo, every), what=f"batch {t}")
+    g.close()
