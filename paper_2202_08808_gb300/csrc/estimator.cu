@@ -252,10 +252,12 @@ static_assert(ER_ROWS == 32 && ER_ROWS / 2 * EST_HID / 4 == ER_NT, "k_est_rows' 
 // of dz1 by the inputs, 8 of h2 by d) and streams those columns through
 // shared memory, ES_ST stages of ES_R rows by asynchronous copies of its
 // warps 2 and 3; 144 blocks keep every SM but a few busy.  What bounds it is the chain of one
-// multiply-add after the other (4096 rows: 16 us, 8 cycles a row); the loads
-// of a thread per parameter straight from row-major arrays made that chain
-// 13 times longer (32 steps of 4096 rows and the loss of 32768: 7.7 ms, 0.84
-// ms now, of which this kernel 0.53).  With lr > 0 the
+// multiply-add after the other: 4.3 cycles a row out of registers, 4.4 out of
+// shared memory with the stage's loop unrolled, 6.2 with two rounds of it (a
+// warp alone).  The loads of a thread per parameter straight from row-major
+// arrays made it 13 times as long (32 steps of 4096 rows and the loss of
+// 32768: 7.7 ms, 0.84 ms with the loop not unrolled, 0.73 now).  Stages of
+// 128 or 512 rows (0.79 and 0.85 ms) and 6 of them (0.87) are slower.  With lr > 0 the
 // parameter's owner then makes the step and its bfloat16 copy.
 constexpr int ES_NT = 128;
 constexpr int ES_R = 256;
@@ -348,14 +350,16 @@ k_est_step(EstCols C, int64_t n, float lr, float *grad, float *master, uint16_t 
             const float *B = ib < 0 ? ones : sm + (s % ES_ST) * ES_MAXC * ES_LD + ib * ES_LD;
             const int rows = (int)(n - s * ES_R < ES_R ? n - s * ES_R : ES_R);
             int r = 0;
-            if (rows == ES_R) {  // 16 rows at a time, the next 16 loaded meanwhile (64 cycles of the chain)
+            // 16 rows at a time, the next 16 loaded meanwhile (64 cycles of the chain); unrolled over the whole
+            // stage, as the copies of the loaded words and the loop's own instructions took a third of the chain
+            if (rows == ES_R) {
                 float4 a[4], q[4];
 #pragma unroll
                 for (int i = 0; i < 4; i++) {
                     a[i] = *(const float4 *)(A + 4 * i);
                     q[i] = *(const float4 *)(B + 4 * i);
                 }
-#pragma unroll 2
+#pragma unroll
                 for (; r < ES_R; r += 16) {
                     float4 a2[4], q2[4];
                     const int nx = r + 16 < ES_R ? r + 16 : 0;
