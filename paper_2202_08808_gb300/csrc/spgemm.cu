@@ -287,7 +287,7 @@ __device__ __forceinline__ void size_long_row(const MatView &A, const MatView &B
 // One thread per row of R sums the B-row lengths of its A entries; rows
 // longer than SIZE_SHORT are listed and summed by a whole warp each (the
 // block's warps share the list), rows longer than SIZE_LONG by the whole
-// block at the end of its round; then the warp hands out bin slots (and,
+// block at the end of its round; then the block hands out bin slots (and,
 // for the static product, the row's place in a fresh C) with one atomic per
 // counter.  A block takes 256 rows a round, or 32 when R has fewer than 32
 // rows a block: a small R of long rows (the hubs a skewed graph's batch
@@ -415,7 +415,8 @@ __global__ void __launch_bounds__(256) k_size_bins(MatView A, MatView B, MatView
         if (b == BIN_CDENSE && (ub > SPLIT_MIN || alen > SPLIT_A) && claim_split(J, ctl, i)) b = -1;
         // Places in the block's share of a bin and of C first, then the block's
         // shares with an atomic each: with an atomic per warp the static
-        // product's 65,536 warps queued at two counters (the kernel 87 us on 2.1 million rows, 59 now, with the wider loads).
+        // product's 65,536 warps queued at two counters (the kernel 87 us on
+        // 2.1 million rows; 59 now, with the wider loads above).
         // A block of 32 rows is one warp's and asks for its places at once.
         const unsigned peers = __match_any_sync(0xffffffffu, b);
         const int leader = __ffs(peers) - 1;
