@@ -73,7 +73,9 @@ typedef struct {
 
 /* An update batch in arrival order (Section 4.1): n entries of
  * (row, col, val, op); val is ignored for DELETE.  Host or device memory
- * per on_device. */
+ * per on_device.  Page-locked host arrays of up to 16384 entries, aligned
+ * to their types, are read by the kernels where they are; others are
+ * copied first. */
 typedef struct {
     int64_t n;
     const int32_t *row;
@@ -235,8 +237,9 @@ dspg_status dspg_apply_batch_algebraic(dspg_handle *h, const dspg_updates *dA, c
  * CSR (rows in order, columns ascending) into caller
  * buffers: rowptr[nrows+1], col[nnz], val[nnz], host or device per
  * on_device (host buffers may be pageable or page-locked; page-locked ones
- * are copied to at full speed).  Two-call convention: with rowptr == NULL
- * only *nnz_out is written.  The handle keeps the read's device scratch
+ * are written at full speed).  Two-call convention: with rowptr == NULL
+ * only *nnz_out is written, and the fill call reuses the row pointers that
+ * call computed while C has not changed in between.  The handle keeps the read's device scratch
  * (up to 256 MiB per buffer) for later reads; a larger read allocates and
  * frees its scratch within the call. */
 dspg_status dspg_read_C(dspg_handle *h, int64_t *nnz_out, int64_t *rowptr, int32_t *col, void *val,
