@@ -6,6 +6,7 @@
 #include <algorithm>
 
 #include "internal.h"
+#include "order_window.h"
 
 namespace dspg {
 
@@ -421,9 +422,11 @@ constexpr int RS_ROWS = 32;        // rows of its tile
 constexpr int RS_PW = RS_ROWS / (RS_NT / 32);  // rows of a warp
 
 // A read may run while an asynchronous batch rewrites other rows of C, and a
-// read of all of C then meets rows that change under it: their entries come
-// out undefined, but every access stays inside the arena and the row's
-// stretch of the result, whose lengths (rp) were taken before.
+// read of all of C then meets rows that change under it, or that have been
+// moved to a place whose entries are not written yet: their entries come out
+// undefined, but every access stays inside the arena, the row's stretch of
+// the result, whose lengths (rp) were taken before, and the windows of
+// columns in shared memory (order_window.h).
 __device__ __forceinline__ int64_t row_start(const MatView &M, int64_t r, int64_t len) {
     const int64_t so = M.off[r], most = M.arena_cap - len;
     return so <= most ? so : (most > 0 ? most : 0);
@@ -577,7 +580,6 @@ k_read_short(const int32_t *rows, int64_t n_arg, const long long *n_dev, MatView
 // copied.  With host arrays (out_col) the row is put together in device
 // memory (dst_col, dst_val: it stays in L2) and stored to the host in order.
 constexpr int OL_NT = 512;
-constexpr int OL_W = 1 << 18;          // columns of a window
 // C wider than this: k_sort_long.  A row then takes up to 16 windows of about
 // 2 us each, what the network takes for rows of 512 to 1024 entries.
 constexpr int64_t OL_MAX_COLS = (int64_t)1 << 22;
@@ -624,8 +626,10 @@ k_order_long(const int32_t *rows, MatView M, const int64_t *rp, const int64_t *l
             const int32_t c = mc[e];
             const int32_t nx = e + 1 < len ? mc[e + 1] : INT32_MAX;
             unsorted |= c > nx;
-            mn = min(mn, c);
-            mx = max(mx, c);
+            if (ow_is_column(c, M.ncols)) {  // always, for a row that does not change meanwhile
+                mn = min(mn, c);
+                mx = max(mx, c);
+            }
         }
         mn = __reduce_min_sync(0xffffffffu, mn);
         mx = __reduce_max_sync(0xffffffffu, mx);
@@ -647,13 +651,18 @@ k_order_long(const int32_t *rows, MatView M, const int64_t *rp, const int64_t *l
         }
         mn = s_mn;
         mx = s_mx;
+        if (mn > mx) {  // no column at all: a row that is being written
+            __syncthreads();  // as above
+            continue;
+        }
         uint32_t carry = 0;  // entries of the windows before
-        for (int wb = mn & ~1023; wb <= mx; wb += W) {
-            const int nb = min(W, (mx - wb + 1024) & ~1023) >> 10;  // 1024-column stretches of this window
+        for (int wb = ow_first(mn); wb <= mx; wb += W) {  // mx < M.ncols <= OL_MAX_COLS: no step overflows
+            const int nb = ow_stretches(wb, mx, W);
+            const uint32_t in = (uint32_t)nb * OL_STRETCH;
 #pragma unroll 4
             for (int64_t e = tid; e < len; e += OL_NT) {
-                const uint32_t c = (uint32_t)(mc[e] - wb);
-                if (c < (uint32_t)nb << 10) {
+                const uint32_t c = ow_place(mc[e], wb);
+                if (c < in) {
                     atomicOr(&bm[c >> 5], 1u << (c & 31));
                     atomicAdd(&cnt[c >> 10], 1u);
                 }
@@ -682,8 +691,8 @@ k_order_long(const int32_t *rows, MatView M, const int64_t *rp, const int64_t *l
 #pragma unroll 4
             for (int64_t e = tid; e < len; e += OL_NT) {
                 const int32_t col = mc[e];
-                const uint32_t c = (uint32_t)(col - wb);
-                if (c < (uint32_t)nb << 10) {
+                const uint32_t c = ow_place(col, wb);
+                if (c < in) {
                     const uint32_t o = first[c >> 10] + pre[c >> 5] + __popc(bm[c >> 5] & ((1u << (c & 31)) - 1u));
                     if (o < (uint64_t)len) {  // always, for a row that does not change meanwhile
                         dst_col[lo + o] = col;
