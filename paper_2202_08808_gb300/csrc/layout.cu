@@ -869,7 +869,7 @@ __global__ void k_listed_keys(const int64_t *rowptr, const int64_t *listed, cons
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < E; q += (int64_t)gridDim.x * blockDim.x) {
         const int k = list_of(pre, nl, q);
         const int64_t p = rowptr[listed[k]] + (q - pre[k]);
-        keys[q] = ((uint64_t)k << cb) | (uint32_t)col[p];
+        keys[q] = ow_list_key((uint64_t)k, col[p], cb);
         idx[q] = (uint32_t)q;
     }
 }

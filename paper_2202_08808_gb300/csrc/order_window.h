@@ -36,6 +36,12 @@ DSPG_HD int32_t ow_stretches(int32_t wb, int32_t mx, int32_t W) {
 // The place of v in the window of nb stretches at wb; in it when below nb * OL_STRETCH.
 DSPG_HD uint32_t ow_place(int32_t v, int32_t wb) { return (uint32_t)v - (uint32_t)wb; }
 
+// The key that sorts value v of the k-th listed row: by row first, whatever v
+// holds, so that a row that is being written displaces no entry of another.
+DSPG_HD uint64_t ow_list_key(uint64_t k, int32_t v, int cb) {
+    return k << cb | ((uint32_t)v & (((uint64_t)1 << cb) - 1));
+}
+
 static_assert(OL_STRETCH == 1 << 10 && OL_W % OL_STRETCH == 0, "windows of whole stretches");
 
 }  // namespace dspg

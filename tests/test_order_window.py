@@ -1,7 +1,8 @@
 """The windows of columns that a read puts a long row in order by
 (order_window.h), run on the host: any 32-bit values whatever leave every mark
 inside the window's shared memory and end the loop over the windows, and a
-row's distinct columns get their places in column order."""
+row's distinct columns get their places in column order.  The keys of rows
+sorted together sort by row first, whatever a value holds."""
 
 import ctypes
 import os
@@ -57,17 +58,23 @@ extern "C" int order_row(const int32_t *v, int64_t len, int64_t ncols, int64_t *
     }
     return 0;
 }
+extern "C" uint64_t list_key(uint64_t k, int32_t v, int cb) { return ow_list_key(k, v, cb); }
 """
 
 
 @pytest.fixture(scope="module")
-def order_row(tmp_path_factory):
+def driver(tmp_path_factory):
     d = tmp_path_factory.mktemp("order_window")
     src, lib = d / "driver.cpp", d / "driver.so"
     src.write_text(DRIVER)
     subprocess.run(["g++", "-O1", "-std=c++17", "-Wall", "-Werror", "-fwrapv", "-fPIC", "-shared", "-I", CSRC, "-o", str(lib),
                     str(src)], check=True)
-    f = ctypes.CDLL(str(lib)).order_row
+    return ctypes.CDLL(str(lib))
+
+
+@pytest.fixture(scope="module")
+def order_row(driver):
+    f = driver.order_row
 
     def call(v, ncols):
         v = np.ascontiguousarray(v, np.int32)
@@ -105,3 +112,15 @@ def test_columns_get_their_places_in_order(order_row, ncols):
         rc, place, _ = order_row(v, ncols)
         assert rc == 0
         assert np.array_equal(place, np.argsort(np.argsort(v)))
+
+
+@pytest.mark.parametrize("cb", [1, 23, 31])
+def test_keys_sort_by_row_first(driver, cb):
+    f = driver.list_key
+    f.restype = ctypes.c_uint64
+    for k in (0, 1, 5, (1 << 16) - 1):
+        for v in EDGES + [(1 << cb) - 1, 1 << (cb - 1)]:
+            key = f(ctypes.c_uint64(k), ctypes.c_int32(v), cb)
+            assert key >> cb == k
+            if 0 <= v < 1 << cb:
+                assert key & ((1 << cb) - 1) == v
