@@ -239,9 +239,11 @@ dspg_status dspg_apply_batch_algebraic(dspg_handle *h, const dspg_updates *dA, c
  * on_device (host buffers may be pageable or page-locked; page-locked ones
  * are written at full speed).  Two-call convention: with rowptr == NULL
  * only *nnz_out is written, and the fill call reuses the row pointers that
- * call computed while C has not changed in between.  The handle keeps the read's device scratch
- * (up to 256 MiB per buffer) for later reads; a larger read allocates and
- * frees its scratch within the call. */
+ * call computed while C has not changed in between (a batch, also
+ * dspg_apply_batch_async and dspg_apply_batch_wait each, counts as a change).
+ * The handle keeps the read's device scratch (up to 256 MiB per buffer) for
+ * later reads; a larger read allocates and frees its scratch within the
+ * call. */
 dspg_status dspg_read_C(dspg_handle *h, int64_t *nnz_out, int64_t *rowptr, int32_t *col, void *val,
                         int on_device, void *stream);
 

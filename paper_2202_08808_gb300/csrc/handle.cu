@@ -2466,6 +2466,10 @@ dspg_status dspg_apply_batch_wait(dspg_handle *h, dspg_batch_stats *stats, void 
     try {
         const cudaStream_t s = (cudaStream_t)stream;
         h->pending = false;
+        // C is the batch's from here on: what a count call found while it ran
+        // (lengths that were changing, or that a rerun below replaces) serves
+        // no fill call any more
+        h->c_serial++;
         try {
             CK(cudaStreamSynchronize(s));
             if (h->prof) stage_times_from_events(h);

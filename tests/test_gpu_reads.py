@@ -106,6 +106,56 @@ def test_fill_call_takes_the_row_pointers_of_its_count_call_only(dspg):
     g.close()
 
 
+@pytest.mark.parametrize("listed", [False, True])
+def test_a_count_call_before_the_wait_does_not_serve_a_fill_after_it(dspg, listed):
+    """The count call of a read made while an asynchronous batch is in flight
+    (the batch's stream idle, so that nothing changes meanwhile): the fill call
+    after the wait scans the lengths again, and when the wait has rerun the
+    batch in larger arenas, returns C after that."""
+    import ctypes
+    import torch
+    from workloads import random_batch, random_csr
+    sr = MIN_PLUS_I32
+    n = 400
+    lib = dspg.load()
+    some = np.random.default_rng(5).permutation(n)[:150].astype(np.int32)
+    every = some if listed else np.arange(n, dtype=np.int32)
+
+    def read(g, nnz, *out):
+        if listed:
+            assert lib.dspg_read_rows_C(g._h, some.ctypes.data, some.size, ctypes.byref(nnz), *out, 0, None) == 0
+        else:
+            assert lib.dspg_read_C(g._h, ctypes.byref(nnz), *out, 0, None) == 0
+
+    for tight in (False, True):
+        A = random_csr(n, n, 10, 31, sr)
+        g = dspg.DynamicSpGEMM(A, **(dict(slack_min=0, slack_div=1 << 20, arena_headroom=1.0) if tight else {}))
+        Ao = OMat.from_csr(A)
+        nnz, grown = ctypes.c_int64(), 0
+        rp, col, val = np.zeros(every.size + 1, np.int64), np.zeros(n * n, np.int32), np.zeros(n * n, np.int32)
+        out = (rp.ctypes.data, col.ctypes.data, val.ctypes.data)
+
+        def fill_launches():
+            k = lib.dspg_kernel_launches()
+            read(g, nnz, *out)
+            k = lib.dspg_kernel_launches() - k
+            assert_rows_match(rp, col[: rp[-1]], val[: rp[-1]], *Ao.multiply_rows(Ao, every), what=f"tight {tight}")
+            return k
+
+        for t in range(3):
+            read(g, nnz, None, None, None)
+            with_kept = fill_launches()
+            b = random_batch(n, n, 3000 if tight else 60, 60 + t, sr, A=Ao.to_csr(), hit_frac=0.1)
+            g.apply_batch_async(b)
+            torch.cuda.synchronize()
+            read(g, nnz, None, None, None)
+            grown += g.apply_batch_wait()["compactions"]
+            Ao.apply(b)
+            assert fill_launches() > with_kept
+        assert (grown > 0) == tight
+        g.close()
+
+
 @pytest.mark.parametrize("nr", [1, 3, 1023, 1025, 4095, 4096, 4097, 9000])
 def test_affected_rows_around_the_one_block_read(dspg, nr):
     """R and its row pointers come from one block up to 4096 rows and from many
