@@ -29,6 +29,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "estimator.cuh"
+#include "host_view.h"
 #include "internal.h"
 
 using namespace dspg;
@@ -1143,13 +1144,16 @@ void upload(dspg_handle *h, UpdWs &w, const dspg_updates *u, BatchIn &in, int k,
     const int32_t *ur = swap ? u->col : u->row, *uc = swap ? u->row : u->col;
     // a short batch in page-locked memory is read in place too, over the C2C
     // link, by the sort (its one reader), if its arrays are aligned for loads
+    // and page-locked from their first byte to their last
     const void *dr = nullptr, *dc = nullptr, *dv = nullptr, *dp = nullptr;
     const bool aligned = ((uintptr_t)ur | (uintptr_t)uc) % sizeof(int32_t) == 0 && (uintptr_t)u->val % h->vsize == 0;
     if (!u->on_device && in.n <= kInPlace && aligned) {
-        dr = device_view(const_cast<int32_t *>(ur));
-        dc = dr ? device_view(const_cast<int32_t *>(uc)) : nullptr;
-        dv = dc ? device_view(const_cast<void *>(u->val)) : nullptr;
-        dp = dv ? device_view(const_cast<uint8_t *>(u->op)) : nullptr;
+        const size_t n = (size_t)in.n;
+        auto view = [](const void *p, size_t bytes) { return range_view(device_view, const_cast<void *>(p), bytes); };
+        dr = view(ur, sizeof(int32_t) * n);
+        dc = dr ? view(uc, sizeof(int32_t) * n) : nullptr;
+        dv = dc ? view(u->val, (size_t)h->vsize * n) : nullptr;
+        dp = dv ? view(u->op, sizeof(uint8_t) * n) : nullptr;
     }
     if (u->on_device) {
         in.row = ur;
