@@ -43,6 +43,14 @@ void ealloc(T **p, size_t n) {
     }
 }
 
+// Device memory of one call.
+struct EBuf {
+    float *p = nullptr;
+    ~EBuf() {
+        if (p) cudaFree(p);
+    }
+};
+
 constexpr int EST_NT = 128;  // threads of a feature block
 
 // What a training step keeps between its kernels, each a column of `ld` rows
@@ -595,7 +603,14 @@ dspg_status dspg_estimator_predict(dspg_estimator *e, const float *X, int64_t n,
     try {
         check_rows(X, n);
         cudaStream_t s = (cudaStream_t)stream;
-        run_rows(e, X, nullptr, n, out, false, 0.0f, false, s);
+        // outputs over the inputs: a block stores its tile's while others have
+        // theirs to read, so they go through memory of their own
+        const uintptr_t x0 = (uintptr_t)X, o0 = (uintptr_t)out;
+        const bool over = o0 < x0 + sizeof(float) * EST_IN * n && x0 < o0 + sizeof(float) * n;
+        EBuf o;
+        if (over) ealloc(&o.p, (size_t)n);
+        run_rows(e, X, nullptr, n, over ? o.p : out, false, 0.0f, false, s);
+        if (over) ECK(cudaMemcpyAsync(out, o.p, sizeof(float) * n, cudaMemcpyDeviceToDevice, s));
         ECK(cudaGetLastError());
         ECK(cudaStreamSynchronize(s));
         return DSPG_OK;

@@ -29,3 +29,20 @@ def test_output_and_gradient_at_tile_edges(dspg, n):
     loss2, g2 = est.grad(X, y)
     assert loss2 == loss and np.array_equal(g, g2)  # every sum has a fixed order
     est.close()
+
+
+@pytest.mark.parametrize("at", [0, 1, 3])
+def test_outputs_over_their_inputs(dspg, at):
+    """dspg_estimator_predict into memory that its inputs lie in: from the
+    first row on, inside, and over the last quarter."""
+    import torch
+    n = 40000
+    rng = np.random.default_rng(at)
+    X = torch.from_numpy(np.log2(1 + rng.integers(0, 5000, (n, 4))).astype(np.float32)).cuda()
+    est = dspg.Estimator(mlp_init_params(7).astype(np.float32))
+    want = est.predict(X)
+    out = X.reshape(-1)[at * n:][:n]
+    torch.cuda.synchronize()
+    assert dspg.load().dspg_estimator_predict(est._e, X.data_ptr(), n, out.data_ptr(), None) == 0
+    assert torch.equal(out, want)
+    est.close()
