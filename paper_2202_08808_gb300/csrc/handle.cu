@@ -729,11 +729,15 @@ void ensure_c_ws(dspg_handle *h, cudaStream_t s) {
         int ctas = (int)std::min<double>(2.0 * h->num_sms, std::max(4.0, budget / per));
         w.gd_ctas = std::max(1, ctas);
         w.gd_acc.reserve(w.gd_w * w.gd_ctas * h->vsize);
-        w.gd_mask.reserve(w.gd_w / 32 * w.gd_ctas);
-        const int64_t nsum = (w.gd_w / 32 + 31) / 32;
-        w.gd_sum.reserve(nsum * w.gd_ctas);
-        CK(cudaMemsetAsync(w.gd_sum.p, 0, sizeof(uint32_t) * nsum * w.gd_ctas, s));
-        init_dense_scratch(h->sr, w.gd_acc.p, w.gd_mask.p, w.gd_w * w.gd_ctas, w.gd_w / 32 * w.gd_ctas, s);
+        int64_t words = 0;
+        if (!gd_direct(w.gd_w)) {
+            words = w.gd_w / 32 * w.gd_ctas;
+            w.gd_mask.reserve(words);
+            const int64_t nsum = (w.gd_w / 32 + 31) / 32;
+            w.gd_sum.reserve(nsum * w.gd_ctas);
+            CK(cudaMemsetAsync(w.gd_sum.p, 0, sizeof(uint32_t) * nsum * w.gd_ctas, s));
+        }
+        init_dense_scratch(h->sr, w.gd_acc.p, w.gd_mask.p, w.gd_w * w.gd_ctas, words, s);
     }
 }
 

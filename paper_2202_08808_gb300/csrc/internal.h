@@ -66,13 +66,18 @@ struct DetectBufs {
 };
 
 // The recompute of rows of C (static build: all rows).
+// The global dense kernel keeps a row's presence bits in shared memory up to
+// this many words (512K columns, 64 KB), beyond that in global memory.
+constexpr int64_t GD_DIRECT = 16384;
+inline bool gd_direct(int64_t gd_w) { return gd_w / 32 <= GD_DIRECT; }
+
 struct CJob {
     const int32_t *R;         // rows to recompute
     int32_t *bins;            // NBINS lists of rows of C, bin_cap each
     int64_t bin_cap;
     void *gd_acc;             // per-CTA dense accumulators (global), gd_w entries each
-    uint32_t *gd_mask;        // per-CTA presence bits, gd_w / 32 words each
-    uint32_t *gd_sum;         // per-CTA summary: bit w set when mask word w is touched, gd_w / 1024 words each
+    uint32_t *gd_mask;        // per-CTA presence bits, gd_w / 32 words each (null: in shared memory, gd_direct)
+    uint32_t *gd_sum;         // per-CTA summary: bit w set when mask word w is touched, gd_w / 1024 words each (or null)
     int64_t gd_w;
     int gd_ctas;
     int64_t m;                // columns of C

@@ -1605,13 +1605,10 @@ k_num_cluster_hash(MatView A, MatView B, MatView C, CJob J, Ctl *ctl, unsigned e
 
 // ------------------------------------------------- global dense kernel
 
-// Up to this many mask words (512K columns) the row's mask lies in shared
-// memory (64 KB) and the read-out goes over all of it, a warp per 32 words,
-// 32 columns at a time: the accumulator is read and cleared in whole lines.
-// Wider rows keep the mask in global memory and go through the summary of
-// touched words.
-constexpr int GD_DIRECT = 16384;
-
+// DIRECT (gd_direct): the row's mask lies in shared memory and the read-out
+// goes over all of it, a warp per 32 words, 32 columns at a time: the
+// accumulator is read and cleared in whole lines.  Wider rows keep the mask
+// in global memory and go through the summary of touched words.
 template <int SR, bool DIRECT>
 __global__ void __launch_bounds__(512)
 k_num_gdense(MatView A, MatView B, MatView C, CJob J, Ctl *ctl, unsigned mask, int bin) {
@@ -2376,7 +2373,7 @@ static void run_numeric_t(const MatView &A, const MatView &B, const MatView &C, 
     // launched: rows of bins that are off go there.
     {
         const int64_t words = J.gd_w / 32;
-        const bool direct = words <= GD_DIRECT;
+        const bool direct = gd_direct(J.gd_w);
         static bool set_g = false;
         if (!set_g) {
             cudaFuncSetAttribute(k_num_gdense<SR, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
