@@ -897,7 +897,7 @@ void build_transpose(dspg_handle *h, cudaStream_t s) {
     const int64_t nnz = mat_rowptr(h, A, nullptr, A.nrows, rowptr.p, s);
     DBuf<int32_t> col;
     col.reserve(nnz + 1);
-    gather_rows_out(nullptr, A.nrows, A.view(), rowptr.p, col.p, nullptr, 0, s, h->num_sms);
+    gather_cols_out(A.nrows, A.view(), rowptr.p, col.p, s, h->num_sms);
     DBuf<uint64_t> k0, k1;
     DBuf<uint32_t> v0, v1, counts;
     DBuf<int64_t> scan_tmp, scan_out;

@@ -283,8 +283,9 @@ void lens_from_rowptr(const int64_t *rowptr, int32_t *len, int64_t n, cudaStream
 void copy_rows(const int32_t *rows, int64_t n, const int64_t *src_off, const int32_t *len, const int32_t *src_col,
                const void *src_val, const int64_t *dst_off, int32_t *dst_col, void *dst_val, int vsize,
                cudaStream_t s, int num_sms);
-void gather_rows_out(const int32_t *rows, int64_t n, const MatView &M, const int64_t *out_rowptr, int32_t *out_col,
-                     void *out_val, int vsize, cudaStream_t s, int num_sms);
+// The columns of M's rows (n of them) at the row pointers out_rowptr.
+void gather_cols_out(int64_t n, const MatView &M, const int64_t *out_rowptr, int32_t *out_col, cudaStream_t s,
+                     int num_sms);
 struct SortScratch {  // for `total` entries: keys, indices (two each), radix counts, scans, gather space
     uint64_t *k0, *k1;
     uint32_t *i0, *i1, *counts;

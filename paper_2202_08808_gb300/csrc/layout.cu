@@ -380,30 +380,21 @@ void copy_rows(const int32_t *rows, int64_t n, const int64_t *src_off, const int
                                                dst_col, (int32_t *)dst_val);
 }
 
-template <typename T>
-__global__ void k_gather_out(const int32_t *rows, int64_t n, MatView M, const int64_t *out_rowptr, int32_t *out_col,
-                             T *out_val) {
+__global__ void k_gather_cols(int64_t n, MatView M, const int64_t *out_rowptr, int32_t *out_col) {
     pdl_begin();
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const T *mv = (const T *)M.val;
-    for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < n; x += nwarps) {
-        const int64_t r = rows ? rows[x] : x;
-        const int64_t so = M.off[r], d = out_rowptr[x];
+    for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n; r += nwarps) {
+        const int64_t so = M.off[r], d = out_rowptr[r];
         const int L = M.len[r];
-        for (int e = lane; e < L; e += 32) {
-            out_col[d + e] = M.col[so + e];
-            if (out_val) out_val[d + e] = mv[so + e];
-        }
+        for (int e = lane; e < L; e += 32) out_col[d + e] = M.col[so + e];
     }
 }
 
-void gather_rows_out(const int32_t *rows, int64_t n, const MatView &M, const int64_t *out_rowptr, int32_t *out_col,
-                     void *out_val, int vsize, cudaStream_t s, int num_sms) {
+void gather_cols_out(int64_t n, const MatView &M, const int64_t *out_rowptr, int32_t *out_col, cudaStream_t s,
+                     int num_sms) {
     if (n <= 0) return;
-    unsigned g = blocks_for(n * 32, 256, (int64_t)num_sms * 16);
-    if (vsize == 8) launch_k(k_gather_out<double>, g, 256, 0, s, rows, n, M, out_rowptr, out_col, (double *)out_val);
-    else launch_k(k_gather_out<int32_t>, g, 256, 0, s, rows, n, M, out_rowptr, out_col, (int32_t *)out_val);
+    launch_k(k_gather_cols, blocks_for(n * 32, 256, (int64_t)num_sms * 16), 256, 0, s, n, M, out_rowptr, out_col);
 }
 
 // ------------------------------------------------- rows out, in column order
