@@ -553,6 +553,32 @@ k_read_short(const int32_t *rows, int64_t n_arg, const long long *n_dev, MatView
     }
 }
 
+// Bitonic sort by column of the N (a power of two) keys in sk, with their
+// values in sv when hv, in the block's shared memory (padding keys INT32_MAX).
+template <typename T>
+__device__ __forceinline__ void block_sort_row(int32_t *sk, T *sv, int N, bool hv) {
+    const int tid = threadIdx.x, nt = blockDim.x;
+    for (int size = 2; size <= N; size <<= 1) {
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            for (int q = tid; q < N / 2; q += nt) {
+                const int a = 2 * q - (q & (stride - 1)), b = a + stride;
+                const bool up = (a & size) == 0;
+                const int32_t ka = sk[a], kb = sk[b];
+                if ((ka > kb) == up) {
+                    sk[a] = kb;
+                    sk[b] = ka;
+                    if (hv) {
+                        const T t = sv[a];
+                        sv[a] = sv[b];
+                        sv[b] = t;
+                    }
+                }
+            }
+            __syncthreads();
+        }
+    }
+}
+
 // The listed rows of more than SORT_SHORT entries, a block each (taken by a
 // ticket, as their lengths differ by orders of magnitude).  The columns of a
 // row are distinct, so the place of an entry in column order is the number
@@ -565,15 +591,23 @@ k_read_short(const int32_t *rows, int64_t n_arg, const long long *n_dev, MatView
 // of two (300-edge batches of R-MAT 18, 27 million entries in rows of 2,000
 // on average into host memory: 4.2 ms with the network in 196 KB of shared
 // memory, one block per SM; 1.55 ms now, the link's rate.  A warp's register
-// network for rows of up to 512 entries measured the same in every case).  Columns are taken in windows of W, from the row's first to its
-// last, and a window keeps 4 blocks of 512 threads on an SM (50 KB at
-// W = 2^18, OL_W).  A row already in order (the dense kernels' rows) is
-// copied.  With host arrays (out_col) the row is put together in device
-// memory (dst_col, dst_val: it stays in L2) and stored to the host in order.
+// network for rows of up to 512 entries measured the same there).  Columns
+// are taken in windows of W, from the row's first to its last, and a window
+// keeps 4 blocks of 512 threads on an SM (50 KB at W = 2^18, OL_W).  A window
+// takes about 3 us however few of the row's columns lie in it, so a short row
+// over several of them goes through a network in the bitmap's memory instead
+// (ow_by_network; 20,000 rows of 72 entries in a C of 2^22 columns: 831 us
+// with the network in 196 KB, 1929 by windows, 250 so).  A row already in
+// order (the dense kernels' rows) is copied.  With host arrays (out_col) the
+// row is put together in device memory (dst_col, dst_val: it stays in L2) and
+// stored to the host in order.
 constexpr int OL_NT = 512;
-// C wider than this: k_sort_long.  A row then takes up to 16 windows of about
-// 2 us each, what the network takes for rows of 512 to 1024 entries.
+// C wider than this: k_sort_long.  At this width 5000 rows of 6000 entries take
+// 2.1 ms by their 16 windows and 4.1 by the network in 196 KB; at twice the
+// width the windows would take as long.
 constexpr int64_t OL_MAX_COLS = (int64_t)1 << 22;
+
+static_assert(2 * OL_NET <= OL_W / 32, "the network's columns and places fit the bitmap of a whole window");
 
 static size_t order_long_smem(int W) { return (size_t)W / 32 * 6 + (size_t)W / 1024 * 8; }
 
@@ -646,6 +680,27 @@ k_order_long(const int32_t *rows, MatView M, const int64_t *rp, const int64_t *l
             __syncthreads();  // as above
             continue;
         }
+        if (ow_by_network(len, (mx - ow_first(mn)) / W + 1)) {
+            int N = 128;
+            while (N < len) N <<= 1;
+            int32_t *sk = (int32_t *)bm, *se = sk + N;  // columns, and where in the row they are
+            for (int e = tid; e < N; e += OL_NT) {
+                sk[e] = e < len ? mc[e] : INT32_MAX;
+                se[e] = e < len ? e : 0;
+            }
+            __syncthreads();
+            block_sort_row<int32_t>(sk, se, N, true);
+            int32_t *oc = out_col ? out_col : dst_col;
+            T *ov = out_col ? out_val : dst_val;
+            for (int64_t e = tid - (int64_t)(lo & 31); e < len; e += OL_NT)
+                if (e >= 0) {
+                    oc[lo + e] = sk[e];
+                    if (has_val) ov[lo + e] = mv[so + se[e]];
+                }
+            __syncthreads();
+            for (int q = tid; q < 2 * N; q += OL_NT) bm[q] = 0u;
+            continue;  // the next row's marks follow a barrier
+        }
         uint32_t carry = 0;  // entries of the windows before
         for (int wb = ow_first(mn); wb <= mx; wb += W) {  // mx < M.ncols <= OL_MAX_COLS: no step overflows
             const int nb = ow_stretches(wb, mx, W);
@@ -707,32 +762,6 @@ k_order_long(const int32_t *rows, MatView M, const int64_t *rp, const int64_t *l
                     out_col[lo + e] = __ldcg(dst_col + lo + e);
                     if (has_val) out_val[lo + e] = __ldcg(dst_val + lo + e);
                 }
-        }
-    }
-}
-
-// Bitonic sort by column of the N (a power of two) keys in sk, with their
-// values in sv when hv, in the block's shared memory (padding keys INT32_MAX).
-template <typename T>
-__device__ __forceinline__ void block_sort_row(int32_t *sk, T *sv, int N, bool hv) {
-    const int tid = threadIdx.x, nt = blockDim.x;
-    for (int size = 2; size <= N; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int q = tid; q < N / 2; q += nt) {
-                const int a = 2 * q - (q & (stride - 1)), b = a + stride;
-                const bool up = (a & size) == 0;
-                const int32_t ka = sk[a], kb = sk[b];
-                if ((ka > kb) == up) {
-                    sk[a] = kb;
-                    sk[b] = ka;
-                    if (hv) {
-                        const T t = sv[a];
-                        sv[a] = sv[b];
-                        sv[b] = t;
-                    }
-                }
-            }
-            __syncthreads();
         }
     }
 }

@@ -36,6 +36,20 @@ DSPG_HD int32_t ow_stretches(int32_t wb, int32_t mx, int32_t W) {
 // The place of v in the window of nb stretches at wb; in it when below nb * OL_STRETCH.
 DSPG_HD uint32_t ow_place(int32_t v, int32_t wb) { return (uint32_t)v - (uint32_t)wb; }
 
+// Whether a row of len entries whose columns span that many windows is put in
+// order by a sorting network over its entries instead: up to 256 entries a
+// window, and at most OL_NET.  Each side of the line as measured, 20,000 rows
+// into device memory, us (network / windows, whose cost is nearly that of
+// going over them):
+//    2 windows:  400 entries  490 / 583,   768 entries  923 / 722
+//    4 windows: 1024 entries  950 / 1244, 1536 entries 1973 / 1443
+//    8 windows: 2048 entries 2047 / 2710, 3000 entries 4358 / 3208
+//   16 windows: 2048 entries 2043 / 4442, 4000 entries 4619 / 6408
+constexpr int OL_NET = 4096;
+DSPG_HD bool ow_by_network(int64_t len, int windows) {
+    return windows > 1 && len <= OL_NET && len <= (int64_t)windows << 8;
+}
+
 // The key that sorts value v of the k-th listed row: by row first, whatever v
 // holds, so that a row that is being written displaces no entry of another.
 DSPG_HD uint64_t ow_list_key(uint64_t k, int32_t v, int cb) {

@@ -9,10 +9,13 @@ import pytest
 
 from oracle import OMat
 from parity import assert_rows_match
-from workloads import CSR, MIN_PLUS_I32, PLUS_TIMES_F64
+from workloads import CSR, MIN_PLUS_I32, OP_SET, PLUS_TIMES_F64, Batch
 
 pytestmark = pytest.mark.gpu
 
+# around the longest rows that go through the network instead of the bitmap's
+# windows: 256 entries a window, at most 4096
+NETWORK = [255, 256, 257, 511, 512, 513, 767, 768, 769, 1023, 1024, 1025, 4095, 4096, 4097]
 LENGTHS = [0, 1, 31, 32, 33, 63, 64, 65, 66, 127, 128, 129, 511, 513, 1025, 2048, 16384, 16385, 20000]
 
 
@@ -27,10 +30,20 @@ def _csr(rows, ncols, sr, rng):
 @pytest.mark.parametrize("sr", [PLUS_TIMES_F64, MIN_PLUS_I32])
 @pytest.mark.parametrize("m", [20480, (1 << 18), (1 << 18) + 1, 600001, (1 << 22) + 33])
 def test_rows_in_order_at_every_width(dspg, m, sr):
+    _rows_in_order(dspg, m, sr, LENGTHS)
+
+
+@pytest.mark.parametrize("sr", [PLUS_TIMES_F64, MIN_PLUS_I32])
+@pytest.mark.parametrize("m", [1 << 18, (1 << 18) + 1, 600001, 1 << 20, 1 << 22])
+def test_rows_in_order_by_network_and_by_windows(dspg, m, sr):
+    _rows_in_order(dspg, m, sr, NETWORK)
+
+
+def _rows_in_order(dspg, m, sr, lengths):
     rng = np.random.default_rng(m + sr)
     edges = np.array([c for c in (0, 1, 1023, 1024, (1 << 18) - 1, 1 << 18, (1 << 18) + 1, m - 2, m - 1) if c < m])
     brows, arows = [], []
-    for length in LENGTHS:
+    for length in lengths:
         cols = np.unique(np.concatenate([edges[: max(0, length // 8)], rng.choice(m, size=length, replace=False)]))
         cols = rng.permutation(cols)[:length]
         # each row of C is the union of disjoint rows of B, so that its columns arrive in runs
@@ -53,6 +66,15 @@ def test_rows_in_order_at_every_width(dspg, m, sr):
     orp, ocol, oval = Ao.multiply_rows(Bo, pick)
     sabs = Ao.multiply_rows(Bo, pick, absval=True)[2] if sr == PLUS_TIMES_F64 else None
     assert_rows_match(*g.read_rows_C(pick), orp, ocol, oval, sabs, "listed rows")
+    first = A.rowptr[:-1]
+    b = Batch(every, A.col[first], A.val[first] + A.val[first], np.full(every.size, OP_SET, np.uint8))
+    g.apply_batch(b)
+    Ao.apply(b)
+    orp, ocol, oval = Ao.multiply_rows(Bo, every)
+    sabs = Ao.multiply_rows(Bo, every, absval=True)[2] if sr == PLUS_TIMES_F64 else None
+    rows, *got = g.read_affected()  # straight into page-locked arrays
+    assert np.array_equal(rows, every)
+    assert_rows_match(*got, orp, ocol, oval, sabs, "affected rows")
     g.close()
 
 
@@ -161,7 +183,6 @@ def test_affected_rows_around_the_one_block_read(dspg, nr):
     """R and its row pointers come from one block up to 4096 rows and from many
     beyond: both one-call reads, with R spread over the bitmap's chunks."""
     import torch
-    from workloads import OP_SET, Batch
     rng = np.random.default_rng(nr)
     n, k, m = 30000, 150, 40
     A = _csr([rng.choice(k, size=int(rng.integers(0, 4)), replace=False) for _ in range(n)], k, MIN_PLUS_I32, rng)
