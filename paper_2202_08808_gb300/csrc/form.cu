@@ -35,15 +35,17 @@ __global__ void k_permute_entries(const uint32_t *idx, const uint32_t *row_of, c
 }
 
 // A warp per output row: |P_i u X_i| = len(P_i) + len(X_i) - |P_i n X_i|.
-__global__ void k_form_count(const int32_t *rows, int64_t n, MatView P, const int64_t *xrp, const int32_t *xcol,
-                             int64_t *cnt) {
+// listed: P holds the listed rows only, row rows[t] as its row t.
+__global__ void k_form_count(const int32_t *rows, int64_t n, MatView P, bool listed, const int64_t *xrp,
+                             const int32_t *xcol, int64_t *cnt) {
     pdl_begin();
     const int lane = threadIdx.x & 31;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < n; t += nw) {
         const int32_t i = rows ? rows[t] : (int32_t)t;
-        const int64_t po = P.off[i];
-        const int pl = P.len[i];
+        const int64_t pi = listed ? t : i;
+        const int64_t po = P.off[pi];
+        const int pl = P.len[pi];
         const int64_t x0 = xrp[i], x1 = xrp[i + 1];
         int both = 0;
         for (int p = lane; p < pl; p += 32) {
@@ -91,7 +93,9 @@ __global__ void k_form_merge(const int32_t *rows, int64_t n, const int64_t *prp,
         int64_t x = xrp[i];
         const int64_t x1 = xrp[i + 1];
         int64_t o = orp[t];
-        while (p < p1 || x < x1) {
+        // the row's room: always enough, but for a row of P that changes while it is read
+        const int64_t o1 = orp[t + 1];
+        while ((p < p1 || x < x1) && o < o1) {
             const int32_t jp = p < p1 ? pcol[p] : 0x7fffffff;
             const int32_t jx = x < x1 ? xcol[x] : 0x7fffffff;
             if (jp == jx) {
@@ -129,10 +133,10 @@ void permute_entries(const uint32_t *idx, const uint32_t *row_of, const void *va
              (char *)out_val, vsize);
 }
 
-void form_count(const int32_t *rows, int64_t n, const MatView &P, const int64_t *xrp, const int32_t *xcol,
+void form_count(const int32_t *rows, int64_t n, const MatView &P, bool listed, const int64_t *xrp, const int32_t *xcol,
                 int64_t *cnt, cudaStream_t s, int num_sms) {
     if (n <= 0) return;
-    launch_k(k_form_count, grid_of(n * 32, 256, num_sms), 256, 0, s, rows, n, P, xrp, xcol, cnt);
+    launch_k(k_form_count, grid_of(n * 32, 256, num_sms), 256, 0, s, rows, n, P, listed, xrp, xcol, cnt);
 }
 
 void form_merge(int sr, const int32_t *rows, int64_t n, const int64_t *prp, const int32_t *pcol, const void *pval,

@@ -444,10 +444,17 @@ struct dspg_handle {
     uint64_t c_serial = 0;
     struct ReadKey {
         bool valid = false;
-        bool all = false;  // every row of C
+        bool all = false;   // every row of C
+        bool form = false;  // row pointers of alpha P (+) beta X (read_form), else of P
         uint64_t serial = 0;
         int64_t nnz = 0;
         std::vector<int32_t> rows;
+        // whether they are those of these rows (NULL: all) of this generation
+        bool serves(uint64_t ser, bool fm, const int32_t *r, int64_t n) const {
+            return valid && serial == ser && form == fm && all == !r &&
+                   (!r || ((int64_t)rows.size() == n &&
+                           (n == 0 || std::memcmp(rows.data(), r, sizeof(int32_t) * (size_t)n) == 0)));
+        }
     } rd_key;
     BatchIn inA, inB;
     InArgs *d_args = nullptr;  // device: where the A, B and forwarded batches are (read by the sorts)
@@ -1458,7 +1465,7 @@ void fill_rows_out(dspg_handle *h, DevMat &M, const MatView &V, int vs, const in
         sort_listed_host(h, M, rp, lh, rph.data(), oc, ov, vs, s);
     };
     if (on_device) {
-        CK(cudaMemcpyAsync(rowptr, rp, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToDevice, s));
+        if (rowptr != rp) CK(cudaMemcpyAsync(rowptr, rp, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToDevice, s));
         rows_out(col, val);
     } else {
         DBuf<int32_t> c_l;
@@ -1494,10 +1501,7 @@ int64_t read_mat(dspg_handle *h, DevMat &M, const int32_t *rows_in, int64_t nr, 
     // again, or all of them), are still in the kept buffer
     dspg_handle::ReadKey &key = h->rd_key;
     const bool keyed = &M == &h->C && (!rows_in || !on_device);
-    const bool hit = keyed && key.valid && key.serial == h->c_serial && key.all == !rows_in &&
-                     (rows_in ? (int64_t)key.rows.size() == n &&
-                                    (n == 0 || std::memcmp(key.rows.data(), rows_in, sizeof(int32_t) * (size_t)n) == 0)
-                              : rowptr != nullptr);
+    const bool hit = keyed && key.serves(h->c_serial, false, rows_in, n) && (rows_in || rowptr);
     key.valid = false;  // the kept row list and row pointers are rewritten below unless this is a hit
     DBuf<int64_t> rp_l;
     int64_t *rp;
@@ -1521,6 +1525,7 @@ int64_t read_mat(dspg_handle *h, DevMat &M, const int32_t *rows_in, int64_t nr, 
     if (keyed && rp == h->rd.rp.p && (rows_in ? rows == h->rd.rows.p : !rowptr)) {
         if (rows_in && !hit) key.rows.assign(rows_in, rows_in + n);
         key.all = !rows_in;
+        key.form = false;
         key.serial = h->c_serial;
         key.nnz = nnz;
         key.valid = true;
@@ -1546,10 +1551,6 @@ int64_t read_form(dspg_handle *h, const int32_t *rows_in, int64_t nr, int64_t *r
             rows = rows_d.p;
         }
     }
-    DBuf<int64_t> cnt, orp, tmp;
-    cnt.reserve(std::max<int64_t>(n, 1));
-    orp.reserve(n + 1);
-    tmp.reserve(scan_tmp_entries(n) + 1);
     const int64_t *xrp = h->has_x ? h->xrp.p : nullptr;
     DBuf<int64_t> zrp;  // no X: empty rows
     if (!xrp) {
@@ -1557,19 +1558,59 @@ int64_t read_form(dspg_handle *h, const int32_t *rows_in, int64_t nr, int64_t *r
         CK(cudaMemsetAsync(zrp.p, 0, sizeof(int64_t) * (h->C.nrows + 1), s));
         xrp = zrp.p;
     }
-    form_count(rows, n, h->C.view(), xrp, h->xcol.p, cnt.p, s, h->num_sms);
-    scan_i64(cnt.p, orp.p, n, tmp.p, s);
-    const int64_t nnz = read_i64(orp.p + n, s);
-    if (!rowptr) return nnz;
     // P's rows, canonical, into scratch
     DBuf<int64_t> prp;
     DBuf<int32_t> pcol;
     DBuf<char> pval;
-    prp.reserve(n + 1);
-    const int64_t pn = read_mat(h, h->C, rows, rows ? n : 0, nullptr, nullptr, nullptr, 1, s);
-    pcol.reserve(std::max<int64_t>(pn, 1));
-    pval.reserve(std::max<int64_t>(pn, 1) * h->vsize);
-    read_mat(h, h->C, rows, rows ? n : 0, prp.p, pcol.p, pval.p, 1, s);
+    auto copy_p = [&]() {
+        prp.reserve(n + 1);
+        const int64_t pn = mat_rowptr(h, h->C, rows, n, prp.p, s);
+        pcol.reserve(std::max<int64_t>(pn, 1));
+        pval.reserve(std::max<int64_t>(pn, 1) * h->vsize);
+        fill_rows_out(h, h->C, h->C.view(), h->vsize, rows, n, prp.p, pn, prp.p, pcol.p, pval.p, 1, s);
+    };
+    // the row pointers, or those of the count call (see read_mat): while a
+    // batch rewrites rows of P the caller's arrays have the room of that call
+    dspg_handle::ReadKey &key = h->rd_key;
+    const bool hit = rowptr && (!rows_in || !on_device) && key.serves(h->c_serial, true, rows_in, n);
+    DBuf<int64_t> orp_l;
+    int64_t nnz;
+    if (hit) {
+        nnz = key.nnz;
+        copy_p();
+    } else {
+        key.valid = false;  // the kept row pointers are rewritten
+        DBuf<int64_t> cnt, tmp;
+        cnt.reserve(std::max<int64_t>(n, 1));
+        tmp.reserve(scan_tmp_entries(n) + 1);
+        DBuf<int32_t> plen;
+        MatView P = h->C.view();
+        if (h->pending) {  // sized by a copy: rows of P change, but a copy's lengths and places agree
+            copy_p();
+            plen.reserve(std::max<int64_t>(n, 1));
+            lens_from_rowptr(prp.p, plen.p, n, s);
+            P.off = prp.p;
+            P.len = plen.p;
+            P.col = pcol.p;
+        }
+        int64_t *orp = read_scratch(h->rd.rp, orp_l, n + 1);
+        form_count(rows, n, P, h->pending, xrp, h->xcol.p, cnt.p, s, h->num_sms);
+        scan_i64(cnt.p, orp, n, tmp.p, s);
+        nnz = read_i64(orp + n, s);
+        if (!rowptr) {
+            if ((!rows_in || !on_device) && orp == h->rd.rp.p) {
+                key.rows.assign(rows_in, rows_in ? rows_in + n : rows_in);
+                key.all = !rows_in;
+                key.form = true;
+                key.serial = h->c_serial;
+                key.nnz = nnz;
+                key.valid = true;
+            }
+            return nnz;
+        }
+        if (!h->pending) copy_p();
+    }
+    const int64_t *orp = orp_l.p ? orp_l.p : h->rd.rp.p;
     DBuf<int32_t> ocol_l;
     DBuf<char> oval_l;
     int32_t *ocol = col;
@@ -1580,12 +1621,12 @@ int64_t read_form(dspg_handle *h, const int32_t *rows_in, int64_t nr, int64_t *r
         ocol = ocol_l.p;
         oval = oval_l.p;
     }
-    form_merge(h->sr, rows, n, prp.p, pcol.p, pval.p, xrp, h->xcol.p, h->xval.p, orp.p, ocol, oval, h->fs, s,
+    form_merge(h->sr, rows, n, prp.p, pcol.p, pval.p, xrp, h->xcol.p, h->xval.p, orp, ocol, oval, h->fs, s,
                h->num_sms);
     if (on_device) {
-        CK(cudaMemcpyAsync(rowptr, orp.p, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToDevice, s));
+        CK(cudaMemcpyAsync(rowptr, orp, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToDevice, s));
     } else {
-        CK(cudaMemcpyAsync(rowptr, orp.p, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToHost, s));
+        CK(cudaMemcpyAsync(rowptr, orp, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToHost, s));
         if (nnz > 0) {
             if (col) CK(cudaMemcpyAsync(col, ocol, sizeof(int32_t) * nnz, cudaMemcpyDeviceToHost, s));
             if (val) CK(cudaMemcpyAsync(val, oval, (size_t)h->vsize * nnz, cudaMemcpyDeviceToHost, s));

@@ -243,7 +243,8 @@ struct FormScalars {
 };
 void permute_entries(const uint32_t *idx, const uint32_t *row_of, const void *val, int64_t nnz, int32_t *out_col,
                      void *out_val, int vsize, cudaStream_t s, int num_sms);
-void form_count(const int32_t *rows, int64_t n, const MatView &P, const int64_t *xrp, const int32_t *xcol,
+// listed: P holds the listed rows only, row rows[t] as its row t
+void form_count(const int32_t *rows, int64_t n, const MatView &P, bool listed, const int64_t *xrp, const int32_t *xcol,
                 int64_t *cnt, cudaStream_t s, int num_sms);
 void form_merge(int sr, const int32_t *rows, int64_t n, const int64_t *prp, const int32_t *pcol, const void *pval,
                 const int64_t *xrp, const int32_t *xcol, const void *xval, const int64_t *orp, int32_t *ocol,

@@ -151,6 +151,59 @@ def test_transposed_gram_with_form(dspg):
     _check(g, Ao, None, 1, 0, sr, 0.5, 2.0, X, "after a batch")
 
 
+@pytest.mark.parametrize("sr", [PLUS_TIMES_F64, MIN_PLUS_I32])
+def test_reads_of_a_form_while_an_asynchronous_batch_runs(dspg, sr):
+    """Reads of alpha A B (+) beta X while a batch rewrites rows of A B (rows of
+    C without slack, so that grown ones move): the rows the batch cannot change
+    come out whole, read together or listed, and reads after the wait, whose
+    count call came before it, are right."""
+    import ctypes
+    import torch
+    A = random_csr(900, 700, 6, 71, sr, empty_frac=0.1)
+    B = random_csr(700, 800, 20, 72, sr, empty_frac=0.1)
+    X = random_csr(900, 800, 4, 73, sr, empty_frac=0.2)
+    alpha, beta = (2.5, -0.75) if sr == PLUS_TIMES_F64 else (3, 5)
+    g = dspg.DynamicSpGEMM(A, B, alpha=alpha, beta=beta, X=X, slack_min=0, slack_div=1 << 20, arena_headroom=4.0)
+    Ao, Bo = OMat.from_csr(A), OMat.from_csr(B)
+    lib, n = dspg.load(), A.nrows
+    every = np.arange(n, dtype=np.int32)
+    side = torch.cuda.Stream()
+    moved = 0
+    for t in range(5):
+        pres, val, bound = _expected(Ao, Bo, 0, 0, sr, alpha, beta, X)
+
+        def same(i, cols, vals):
+            tol = 1e-12 * bound[i][pres[i]] if sr == PLUS_TIMES_F64 else 0
+            return np.array_equal(cols, np.nonzero(pres[i])[0]) and np.all(np.abs(vals - val[i][pres[i]]) <= tol)
+
+        b = random_batch(n, A.ncols, 150, 74 + t, sr, A=Ao.to_csr())
+        g.apply_batch_async(b)
+        mid = g.read_C(stream=side)
+        rows = np.random.default_rng(t).permutation(every)[:300]
+        listed = g.read_rows_C(rows, stream=side)
+        torch.cuda.synchronize()
+        nnz = ctypes.c_int64()
+        assert lib.dspg_read_C(g._h, ctypes.byref(nnz), None, None, None, 0, None) == 0
+        moved += g.apply_batch_wait()["relocations"]
+        changed = np.zeros(n, bool)
+        changed[g.last_affected()] = True
+        for i in np.nonzero(~changed)[0]:
+            lo, hi = mid.rowptr[i], mid.rowptr[i + 1]
+            assert same(i, mid.col[lo:hi], mid.val[lo:hi]), f"batch {t}: row {i}"
+        rp, col, v = listed
+        for k, i in enumerate(rows):
+            if not changed[i]:
+                assert same(i, col[rp[k]:rp[k + 1]], v[rp[k]:rp[k + 1]]), f"batch {t}: listed row {i}"
+        Ao.apply(b)
+        pres, val, bound = _expected(Ao, Bo, 0, 0, sr, alpha, beta, X)
+        rp, col, v = np.zeros(n + 1, np.int64), np.zeros(n * 800, np.int32), np.zeros(n * 800, A.val.dtype)
+        assert lib.dspg_read_C(g._h, ctypes.byref(nnz), rp.ctypes.data, col.ctypes.data, v.ctypes.data, 0, None) == 0
+        for i in every:
+            assert same(i, col[rp[i]:rp[i + 1]], v[rp[i]:rp[i + 1]]), f"batch {t}: row {i} after the wait"
+    assert moved > 0
+    g.close()
+
+
 def test_form_rejects_bad_shapes(dspg):
     A = random_csr(30, 20, 3, 61, PLUS_TIMES_F64)
     B = random_csr(25, 40, 3, 62, PLUS_TIMES_F64)
