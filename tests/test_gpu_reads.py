@@ -211,7 +211,9 @@ def test_affected_rows_around_the_one_block_read(dspg, nr):
 
 def test_whole_read_while_an_asynchronous_batch_rewrites_rows(dspg):
     """A read of all of C while a batch runs: the rows the batch cannot change
-    come out whole, whatever the others hold, and the next read is right."""
+    come out whole, whatever the others hold, and the next read is right.  The
+    rows of C have no slack, so that rows of more than 64 entries move to the
+    arena's tail, in memory that held other values before."""
     import torch
     from workloads import random_batch
     sr = MIN_PLUS_I32
@@ -219,15 +221,21 @@ def test_whole_read_while_an_asynchronous_batch_rewrites_rows(dspg):
     n, m = 1500, 300000
     A = _csr([rng.choice(n, size=int(rng.integers(0, 30)), replace=False) for _ in range(n)], n, sr, rng)
     B = _csr([rng.choice(m, size=int(rng.integers(0, 200)), replace=False) for _ in range(n)], m, sr, rng)
-    g = dspg.DynamicSpGEMM(A, B)
+    torch.cuda.empty_cache()
+    junk = torch.randint(-2**31, 2**31 - 1, (1 << 28,), dtype=torch.int32, device="cuda")  # 1 GiB, given back
+    torch.cuda.synchronize()
+    del junk
+    torch.cuda.empty_cache()
+    g = dspg.DynamicSpGEMM(A, B, slack_min=0, slack_div=1 << 20, arena_headroom=6.0)
     Ao, Bo = OMat.from_csr(A), OMat.from_csr(B)
     every = np.arange(n, dtype=np.int32)
     side = torch.cuda.Stream()
+    room_a = (np.diff(A.rowptr) + 3) // 4 * 4
     for t in range(6):
         b = random_batch(n, n, 400, 20 + t, sr, A=Ao.to_csr())
         g.apply_batch_async(b)
         mid = g.read_C(stream=side)
-        g.apply_batch_wait()
+        st = g.apply_batch_wait()
         changed = np.zeros(n, bool)
         changed[g.last_affected()] = True
         orp, ocol, oval = Ao.multiply_rows(Bo, every)  # before the batch
@@ -237,5 +245,12 @@ def test_whole_read_while_an_asynchronous_batch_rewrites_rows(dspg):
             assert np.array_equal(mid.val[lo:hi], oval[orp[i]:orp[i + 1]]), f"batch {t}: row {i}"
         Ao.apply(b)
         C = g.read_C()
-        assert_rows_match(C.rowptr, C.col, C.val, *Ao.multiply_rows(Bo, every), what=f"batch {t}")
+        want = Ao.multiply_rows(Bo, every)
+        assert_rows_match(C.rowptr, C.col, C.val, *want, what=f"batch {t}")
+        # of the rows that moved, those that are not A's and not short ones of C that grew are long rows of C
+        len_a = np.diff(Ao.to_csr().rowptr)
+        moved_a = len_a > room_a
+        room_a[moved_a] = (len_a[moved_a] + 3) // 4 * 4
+        short = np.sum((np.diff(want[0]) > np.diff(orp)) & (np.diff(want[0]) <= 64))
+        assert st["relocations"] > moved_a.sum() + short and st["compactions"] == 0
     g.close()
