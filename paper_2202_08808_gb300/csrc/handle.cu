@@ -1442,7 +1442,7 @@ void fill_rows_out(dspg_handle *h, DevMat &M, const MatView &V, int vs, const in
     const int64_t list_cap = nnz / 16385 + 1;
     DBuf<int64_t> long_l, huge_l;
     int64_t *longs = read_scratch(h->rd.long_l, long_l, std::min<int64_t>(n, nnz / 65) + 1);
-    int64_t *huge = read_scratch(h->rd.huge_l, huge_l, list_cap);
+    int64_t *huge = read_has_huge(V.ncols) ? read_scratch(h->rd.huge_l, huge_l, list_cap) : nullptr;
     h->rd.res.reserve(1);
     CK(cudaMemsetAsync(h->rd.res.p, 0, sizeof(ReadOut), s));
     auto rows_out = [&](int32_t *oc, void *ov) {
@@ -2711,7 +2711,7 @@ dspg_status dspg_read_affected_C(dspg_handle *h, int64_t rows_cap, int64_t nnz_c
         }
         if (direct) {
             w.long_l.reserve(std::max<int64_t>(n, 1));
-            w.huge_l.reserve(std::max<int64_t>(n, 1));
+            if (read_has_huge(h->C.ncols)) w.huge_l.reserve(std::max<int64_t>(n, 1));
             w.c.reserve(std::max<int64_t>(nnz_cap, 1));
             w.v.reserve(std::max<int64_t>(nnz_cap, 1) * std::max(h->vsize, 1));
             h->hro->flags = READ_UNORDERED;  // until the read says otherwise
@@ -2807,7 +2807,7 @@ dspg_status dspg_apply_read_affected(dspg_handle *h, const dspg_updates *dA, con
             w.chunk_ex.reserve(nch + 1);
             w.res.reserve(1);
             w.long_l.reserve(rc);
-            w.huge_l.reserve(rc);
+            if (read_has_huge(h->C.ncols)) w.huge_l.reserve(rc);
             w.c.reserve(std::max<int64_t>(nnz_cap, 1));
             w.v.reserve(std::max<int64_t>(nnz_cap, 1) * std::max(h->vsize, 1));
             dspg_batch_stats local;

@@ -330,7 +330,7 @@ enum : unsigned { READ_TOO_SMALL = 1u, READ_UNORDERED = 2u };
 // as the scratch of the longer rows.  The values' array may be null: then
 // columns only.  Lists: one entry per row of more than 64 entries
 // (long_list), and in a C of more than 2^22 columns per row of more than
-// 16384 (huge_list); res zeroed by the caller.  host_res (or null): mapped
+// 16384 (huge_list, else null); res zeroed by the caller.  host_res (or null): mapped
 // host memory that gets what the host needs of res, all but n_huge.
 // n_dev (or null): n read on the device, n then bounding it (grid sizes).
 void read_rows_out(const int32_t *rows, int64_t n, const long long *n_dev, const MatView &M, int vsize,
