@@ -25,7 +25,9 @@
  *  - Indices are int32 (rows, columns), offsets int64.
  *  - Pointers marked "host or device" are device pointers when the
  *    accompanying on_device flag is 1 and host pointers otherwise; they are
- *    only read during the call (borrowed) and copied into library memory.
+ *    borrowed for the call (a batch of dspg_apply_batch_async until its wait
+ *    returns), read where they are or copied into library memory, and not
+ *    kept.
  *  - The handle owns A', B', C' and all working memory on the device; no
  *    pointer into library memory is ever returned.
  *  - All work is enqueued on the given stream (0 = legacy default stream);
@@ -73,9 +75,9 @@ typedef struct {
 
 /* An update batch in arrival order (Section 4.1): n entries of
  * (row, col, val, op); val is ignored for DELETE.  Host or device memory
- * per on_device.  Page-locked host arrays of up to 16384 entries, aligned
- * to their types, are read by the kernels where they are; others are
- * copied first. */
+ * per on_device.  Host arrays of up to 16384 entries that are page-locked
+ * as a whole and aligned to their types are read by the kernels where they
+ * are; others are copied first. */
 typedef struct {
     int64_t n;
     const int32_t *row;

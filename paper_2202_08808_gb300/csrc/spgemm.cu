@@ -1939,9 +1939,10 @@ void run_size_bins(const MatView &A, const MatView &B, const MatView &C, const C
 // (min,+) an accumulator that is not the neutral element has been reached (a
 // sum of two values below 2^30 is never INT32_MAX), in (+,.) a byte is
 // stored.  1000 edges of R-MAT 20 against 256 columns (3.5 million A
-// entries): 132 us with chunks of 2048 entries, the loads one after the other
+// entries): 108.6 us with chunks of 2048 entries, the loads one after the other,
 // an atomic per product on the presence words and every row folded through
-// global memory, 80 us now (SPLIT_END 2 to 16: 316, 320, 329, 337 us a pass).
+// global memory, 64.1 us now (the kernel alone, cold caches; with SPLIT_END 2,
+// 4, 8 and 16 the batch and the read of its rows 316, 320, 329 and 337 us).
 __global__ void __launch_bounds__(1024) k_split_prep(MatView A, CJob J, Ctl *ctl, unsigned mask) {
     pdl_begin();
     __shared__ int incl[1024], wsum[32];
