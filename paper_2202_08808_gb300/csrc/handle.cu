@@ -861,8 +861,16 @@ void static_recompute(dspg_handle *h, cudaStream_t s) {
     const bool exact = h->opt.exact_static == 1 ||
                        (double)need * entry_b * h->opt.arena_headroom > 0.25 * (double)(free_b + C.col.n * entry_b);
     CK(cudaMemsetAsync(&h->ctl->status, 0, sizeof(unsigned), s));
+    // the bins that hold rows: the kernels of the others would only keep the
+    // launches of these waiting (100,000 rows of 81 products: 240 us with the
+    // bins of short rows launched first, 273 with those of long rows first,
+    // 214 so)
+    unsigned long long used = 0;
+    for (int b = 0; b < NBINS; b++)
+        if (h->hctl->bin_count[b] > 0) used |= 1ull << b;
     if (exact) {
         CJob Jc = c_job(h, h->wc.iota.p, true);
+        Jc.bin_on &= used;
         Jc.count_only = 1;
         numeric_branches(h, s, Jc);
         read_ctl(h, s);
@@ -887,7 +895,9 @@ void static_recompute(dspg_handle *h, cudaStream_t s) {
     CK(cudaMemcpyAsync(&h->ctl->n_affected, &nn, sizeof(long long), cudaMemcpyHostToDevice, s));
     // the bins of the sizing pass are still in place; restore their counts
     CK(cudaMemcpyAsync(h->ctl->bin_count, h->hctl->bin_count, sizeof(h->hctl->bin_count), cudaMemcpyHostToDevice, s));
-    numeric_branches(h, s, c_job(h, h->wc.iota.p, true));
+    CJob J = c_job(h, h->wc.iota.p, true);
+    J.bin_on &= used;
+    numeric_branches(h, s, J);
     read_ctl(h, s);
     check_debug(h->hctl);
     if (h->hctl->status & ST_TIMEOUT) throw Err(DSPG_ERR_TIMEOUT, overflow_message(h->hctl));
