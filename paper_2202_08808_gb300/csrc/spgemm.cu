@@ -780,6 +780,11 @@ __device__ __forceinline__ int hash_acc_from(int32_t *keys, T *vals, uint32_t h,
     return -1;  // table full: cannot happen when the bin bound holds
 }
 
+template <int LOG_TS, typename T, int SR>
+__device__ __forceinline__ int hash_acc(int32_t *keys, T *vals, int32_t j, T v) {
+    return hash_acc_from<LOG_TS, T, SR>(keys, vals, ((uint32_t)j * 2654435761u) >> (32 - LOG_TS), j, v);
+}
+
 // Finds or claims the slot of column j.  The product that claims a slot
 // stores its value v there with a plain store, so the table's values need no
 // initial value and only a product whose column is there already needs an
@@ -790,6 +795,20 @@ __device__ __forceinline__ int hash_acc_from(int32_t *keys, T *vals, uint32_t h,
 // compare-and-swap loop around an add of the pipe that is 1/64 as wide as
 // the single-precision one) from 97 of 100 products: the recompute of a
 // 300-edge batch of R-MAT 18 926 to 869 us, its 1024-slot kernel 291 to 232.
+// Where products of one round share columns, the adds that wait for the
+// round meet each other, and what the claims cost is left.  Static products
+// of 30 million products, us with / without claims, for rows whose columns
+// are all different | as many as their products, at random | one block:
+//   group kernels, (+,.), 400 products a row     475 / 796 | 420 / 684 | 326 / 367
+//   group kernels, (min,+), 400                  427 / 433 | 377 / 375 | 260 / 252
+//   8192 slots, (+,.), 7744                      786 / 956 | 522 / 575 | 721 / 611
+//   16384 slots, (+,.), 14400                    789 / 945 | 605 / 656 | 1009 / 835
+//   16384 slots, (min,+), 14400                  771 / 823 | 551 / 565 | 373 / 389
+// So the group kernels of (min,+), whose atomics are native, go without (300
+// edges of a squared R-MAT 18 in (min,+) 1907 to 1877 us); so do the 16384
+// slots of (+,.), which R-MAT batches do not notice (2416 us at scale 18).
+// The 8192 slots keep them: exact sizing of R-MAT 17 is 1030 us with and 1150
+// without.
 template <int LOG_TS, typename T>
 __device__ __forceinline__ int hash_claim(int32_t *keys, T *vals, int32_t j, T v, int &fresh) {
     constexpr int TS = 1 << LOG_TS;
@@ -1289,30 +1308,42 @@ k_num_group_hash(MatView A, MatView B, MatView C, CJob J, Ctl *ctl, unsigned mas
     long long nnz_acc = 0;
     const long long cnt = ctl->bin_count[bin];
     if ((long long)blockIdx.x * NG >= cnt) return;  // no row for this block
+    constexpr bool CLAIMS = SR == SR_PT;  // see hash_claim
+    auto clear = [&](int s) {
+        keys[s] = -1;
+        if (!CLAIMS) vals[s] = Sr<SR>::zero();
+    };
     // the table is cleared once here; each row's read-out clears the slots
     // it used
-    for (int s = gl; s < TS; s += G) keys[s] = -1;
+    for (int s = gl; s < TS; s += G) clear(s);
     __syncwarp(gmask);
     for (long long it = (long long)blockIdx.x * NG + g; it < cnt; it += (long long)gridDim.x * NG) {
         int32_t i = J.bins[(int64_t)bin * J.bin_cap + it];
         if (!dcheck(ctl, i >= 0 && i < A.nrows, DBG_R_ROW, it)) i = 0;  // debug build: a bad list entry fails the batch
         bool ok = true;
         int fresh = 0;  // slots this lane claimed: the row's length, summed over the group
-        group_products<SR, G>(
-            A, B, i, gmask,
-            [&](int32_t j, T v) {
-                const int r = hash_claim<LOG_TS, T>(keys, vals, j, v, fresh);
-                ok &= r != -2;
-                return r;
-            },
-            0, -1, G, [&](int h, T v) { Sr<SR>::acc(&vals[h], v); });
+        if constexpr (CLAIMS)
+            group_products<SR, G>(
+                A, B, i, gmask,
+                [&](int32_t j, T v) {
+                    const int r = hash_claim<LOG_TS, T>(keys, vals, j, v, fresh);
+                    ok &= r != -2;
+                    return r;
+                },
+                0, -1, G, [&](int h, T v) { Sr<SR>::acc(&vals[h], v); });
+        else
+            group_products<SR, G>(A, B, i, gmask, [&](int32_t j, T v) {
+                const int r = hash_acc<LOG_TS, T, SR>(keys, vals, j, v);
+                ok &= r >= 0;
+                fresh += r > 0;
+            });
         const bool full = (__ballot_sync(gmask, !ok) & gmask) != 0u;
         if (full) {
             // a learned table too small: the row goes to the overflow list and
             // is counted and recomputed later; with a bound or exact size a
             // full table cannot happen, so it is reported as an error
             __syncwarp(gmask);
-            for (int s = gl; s < TS; s += G) keys[s] = -1;
+            for (int s = gl; s < TS; s += G) clear(s);
             if (gl == 0) {
                 if (J.sizing == SIZE_LEARNED) J.ovf[atomic_add_ll2(&ctl->n_ovf, 1)] = i;
                 else report_overflow(ctl, bin, i, A, B);
@@ -1333,7 +1364,7 @@ k_num_group_hash(MatView A, MatView B, MatView C, CJob J, Ctl *ctl, unsigned mas
                     const int x = x0 + __popc(bal & ((1u << gl) - 1u));
                     ck[x] = k;
                     cv[x] = vals[s];
-                    keys[s] = -1;
+                    clear(s);
                 }
                 x0 += __popc(bal);
             }
@@ -1368,7 +1399,7 @@ k_num_group_hash(MatView A, MatView B, MatView C, CJob J, Ctl *ctl, unsigned mas
                         C.col[dest + x] = k;
                         Cv[dest + x] = vals[s];
                     }
-                    keys[s] = -1;
+                    clear(s);
                 }
                 x0 += __popc(bal);
             }
@@ -1405,8 +1436,13 @@ k_num_cta_hash(MatView A, MatView B, MatView C, CJob J, Ctl *ctl, unsigned mask,
     long long nnz_acc = 0;
     const long long cnt = ctl->bin_count[bin];
     if (blockIdx.x >= cnt) return;  // no row for this CTA (an empty bin costs no table clear)
+    constexpr bool CLAIMS = SR == SR_MP || LOG_TS < 14;  // see hash_claim
+    auto clear = [&](int s) {
+        keys[s] = -1;
+        if (!CLAIMS) vals[s] = Sr<SR>::zero();
+    };
     // the table is cleared once here; each row's read-out clears the slots it used
-    for (int s = tid; s < TS; s += NT) keys[s] = -1;
+    for (int s = tid; s < TS; s += NT) clear(s);
     if (tid == 0) s_n = 0;
     __syncthreads();
     for (long long it = blockIdx.x; it < cnt; it += gridDim.x) {
@@ -1414,20 +1450,27 @@ k_num_cta_hash(MatView A, MatView B, MatView C, CJob J, Ctl *ctl, unsigned mask,
         if (!dcheck(ctl, i >= 0 && i < A.nrows, DBG_R_ROW, it)) i = 0;  // debug build: a bad list entry fails the batch
         bool ok = true;
         int fresh = 0;  // slots this thread claimed; their sum is the row's length
-        block_products<SR>(
-            A, B, i, ps,
-            [&](int32_t j, T v) {
-                const int r = hash_claim<LOG_TS, T>(keys, vals, j, v, fresh);
-                ok &= r != -2;
-                return r;
-            },
-            0, 1, KeepAll(), [&](int h, T v) { Sr<SR>::acc(&vals[h], v); });
+        if constexpr (CLAIMS)
+            block_products<SR>(
+                A, B, i, ps,
+                [&](int32_t j, T v) {
+                    const int r = hash_claim<LOG_TS, T>(keys, vals, j, v, fresh);
+                    ok &= r != -2;
+                    return r;
+                },
+                0, 1, KeepAll(), [&](int h, T v) { Sr<SR>::acc(&vals[h], v); });
+        else
+            block_products<SR>(A, B, i, ps, [&](int32_t j, T v) {
+                const int r = hash_acc<LOG_TS, T, SR>(keys, vals, j, v);
+                ok &= r >= 0;
+                fresh += r > 0;
+            });
         fresh = warp_sum<int>(fresh);
         if (lane == 0 && fresh) atomicAdd(&s_n, fresh);
         const bool full = __syncthreads_or(!ok);
         const int n = s_n;
         if (full) {  // table too small: see the group kernel
-            for (int s = tid; s < TS; s += NT) keys[s] = -1;
+            for (int s = tid; s < TS; s += NT) clear(s);
             __syncthreads();  // every thread has read s_n
             if (tid == 0) {
                 s_n = 0;
@@ -1462,7 +1505,7 @@ k_num_cta_hash(MatView A, MatView B, MatView C, CJob J, Ctl *ctl, unsigned mask,
                         C.col[dest + x] = k;
                         Cv[dest + x] = vals[s];
                     }
-                    keys[s] = -1;
+                    clear(s);
                 }
             }
         }
