@@ -1975,17 +1975,18 @@ void run_size_bins(const MatView &A, const MatView &B, const MatView &C, const C
 // per-row counter) writes the row into C in column order and resets the
 // accumulator for the next launch.
 // Bound by the gathers of B's row headers and entries (a few per row) from
-// L2.  A warp runs three steps ahead of itself, so that a step waits for one
-// of the three loads that follow one another instead of all of them:
-// the A entries of step t + 2, the B headers of step t + 1 and the B entries
-// of step t are in flight together.  Columns present need no atomic: in
-// (min,+) an accumulator that is not the neutral element has been reached (a
-// sum of two values below 2^30 is never INT32_MAX), in (+,.) a byte is
-// stored.  1000 edges of R-MAT 20 against 256 columns (3.5 million A
-// entries): 108.6 us with chunks of 2048 entries, the loads one after the other,
-// an atomic per product on the presence words and every row folded through
-// global memory, 64.1 us now (the kernel alone, cold caches; with SPLIT_END 2,
-// 4, 8 and 16 the batch and the read of its rows 316, 320, 329 and 337 us).
+// L2.  Columns present need no atomic: in (min,+) an accumulator that is not
+// the neutral element has been reached (a sum of two values below 2^30 is
+// never INT32_MAX), in (+,.) a byte is stored.  1000 edges of R-MAT 20
+// against 256 columns (3.5 million A entries): 108.6 us with chunks of 2048
+// entries, an atomic per product on the presence words and every row folded
+// through global memory, 70.4 us now (the kernel alone, cold caches; with
+// SPLIT_END 2, 4, 8 and 16 the batch and the read of its rows 316, 320, 329
+// and 337 us).  A product loop that loaded the next steps' A entries and B
+// headers ahead took 64.1 (the batch 0.2504 against 0.2520 ms) and 20 to 40
+// percent more than this in (+,.)
+// with 20 entries a row of B (1000 rows of 2000 A entries against 256
+// columns: the static product 595 us with it, 459 without).
 __global__ void __launch_bounds__(1024) k_split_prep(MatView A, CJob J, Ctl *ctl, unsigned mask) {
     pdl_begin();
     __shared__ int incl[1024], wsum[32];
@@ -2006,78 +2007,6 @@ __global__ void __launch_bounds__(1024) k_split_prep(MatView A, CJob J, Ctl *ctl
         __syncthreads();
     }
     if (threadIdx.x == 0) J.sp_pre[cnt] = carry;
-}
-
-// Calls emit(j, a (x) b) for the products of the A entries [a_lo, a_hi) of
-// the row at aoff, this warp taking the groups of 32 from w * 32 in steps of
-// NT; returns the products of this lane's A entries.
-template <int SR, int NT, class F>
-__device__ __forceinline__ long long split_products(const MatView &A, const MatView &B, int64_t aoff, int a_lo, int a_hi,
-                                                    F emit) {
-    using T = typename Sr<SR>::T;
-    constexpr unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const T *Av = (const T *)A.val;
-    const T *Bv = (const T *)B.val;
-    const int first = a_lo + (threadIdx.x >> 5) * 32 + lane;
-    long long prods = 0;
-    // in flight: the A entry of the step after the next (k2, av2), and the next step's B header
-    auto load_a = [&](int ai, int32_t &k, T &av) {
-        k = ai < a_hi ? A.col[aoff + ai] : -1;
-        av = ai < a_hi ? Av[aoff + ai] : T(0);
-    };
-    auto load_b = [&](int32_t k, int64_t &off, int &len) {
-        off = k >= 0 ? B.off[k] : 0;
-        len = k >= 0 ? B.len[k] : 0;
-    };
-    int32_t k1, k2;
-    T av1, av2;
-    load_a(first, k1, av1);
-    load_a(first + NT, k2, av2);
-    int64_t boff;
-    int blen;
-    load_b(k1, boff, blen);
-    for (int ai = first; ai - lane < a_hi; ai += NT) {
-        const T av = av1;
-        const int64_t bo = boff;
-        const int bl = blen;
-        k1 = k2;
-        av1 = av2;
-        load_a(ai + 2 * NT, k2, av2);
-        load_b(k1, boff, blen);
-        prods += bl;
-        int incl = bl;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int o = __shfl_up_sync(FULL, incl, d);
-            if (lane >= d) incl += o;
-        }
-        const int total = __shfl_sync(FULL, incl, 31);
-        const int64_t rel = bo - (incl - bl);  // product p of this lane's entry is B entry rel + p
-        for (int base = 0; base < total; base += 32 * PU) {
-            int32_t c[PU];
-            T v[PU], a[PU];
-#pragma unroll
-            for (int u = 0; u < PU; u++) {
-                const int p = base + u * 32 + lane;
-                int s = 0;
-#pragma unroll
-                for (int step = 16; step > 0; step >>= 1)
-                    if (__shfl_sync(FULL, incl, s + step - 1) <= p) s += step;
-                const int64_t q = __shfl_sync(FULL, rel, s) + p;
-                a[u] = __shfl_sync(FULL, av, s);
-                c[u] = -1;
-                if (p < total) {
-                    c[u] = __ldg(B.col + q);
-                    v[u] = __ldg(Bv + q);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < PU; u++)
-                if (c[u] >= 0) emit(c[u], Sr<SR>::mul(a[u], v[u]));
-        }
-    }
-    return prods;
 }
 
 template <int SR, int NT>
@@ -2131,11 +2060,12 @@ k_num_dsplit(MatView A, MatView B, MatView C, CJob J, Ctl *ctl, unsigned mask, i
         w = end;
         if (c0 >= c1) continue;  // only units that stand for the row's end
         const int pending = c1 - c0;  // this CTA's chunks of the row
-        prods += split_products<SR, NT>(A, B, A.off[i], c0 * SPLIT_CHUNK, c1 == nch ? alen : c1 * SPLIT_CHUNK,
-                                        [&](int32_t j, T v) {
-                                            if (SR == SR_PT) pres[j] = 1;
-                                            Sr<SR>::acc(&acc[j], v);
-                                        });
+        // each warp takes groups of 32 A entries of the chunks (no block barriers)
+        group_products<SR, 32>(A, B, i, 0xffffffffu, [&](int32_t j, T v) {
+            if (SR == SR_PT) pres[j] = 1;
+            Sr<SR>::acc(&acc[j], v);
+            prods++;
+        }, c0 * SPLIT_CHUNK + (tid >> 5) * 32, c1 == nch ? alen : c1 * SPLIT_CHUNK, NT);
         __syncthreads();
         const bool whole = pending == nch;  // nobody else has a part of this row
         T *gacc = (T *)J.sp_acc + slot * mp;
