@@ -2340,37 +2340,56 @@ static void run_numeric_t(const MatView &A, const MatView &B, const MatView &C, 
         launch_s64();
         return;
     }
-    // the longest rows first: a kernel of few long rows leaves room on the
-    // SMs that the bins of shorter rows fill, and nothing long is left for
-    // the end (300-edge batches of R-MAT 18: the recompute 869 us with the
-    // global dense bin last, its mask in global memory, 732 so).  The global dense bin is always
-    // launched: rows of bins that are off go there.
-    {
-        const int64_t words = J.gd_w / 32;
-        const bool direct = gd_direct(J.gd_w);
-        static bool set_g = false;
-        if (!set_g) {
-            cudaFuncSetAttribute(k_num_gdense<SR, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(GD_DIRECT * sizeof(uint32_t)));
-            set_g = true;
+    // Which bins go first.  A kernel of few long rows leaves room on the SMs
+    // for the bins of shorter rows, and nothing long is left for the end when
+    // it starts first; but while no row is long it only delays the kernels
+    // that hold the bulk of the rows.  How long a row can get is what C's
+    // width allows, so the line is drawn there.  Longest first / shortest
+    // first, us, squares of R-MAT graphs: scale 18, a batch of 600 entries 916 /
+    // 965; scale 17, 250 edges and the read 1798 / 1828 in (+,.), 1176 / 1177 in
+    // (min,+); scale 16, 100 edges and the read 712 / 699; scale 15, a batch of
+    // 1000 entries 287 / 280, scale 14 of one entry 114 / 103.  The global dense
+    // bin is always launched: rows of bins that are off go there.
+    auto launch = [&](int bin) {
+        if (bin == BIN_GD) {
+            const bool direct = gd_direct(J.gd_w);
+            static bool set_g = false;
+            if (!set_g) {
+                cudaFuncSetAttribute(k_num_gdense<SR, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(GD_DIRECT * sizeof(uint32_t)));
+                set_g = true;
+            }
+            launch_k(direct ? k_num_gdense<SR, true> : k_num_gdense<SR, false>, grid_for(J.gd_ctas, J.rows_hint, 1), 512,
+                     direct ? (size_t)(J.gd_w / 32) * sizeof(uint32_t) : 0, next(), A, B, C, J, ctl, mask, (int)BIN_GD);
+            return;
         }
-        launch_k(direct ? k_num_gdense<SR, true> : k_num_gdense<SR, false>, grid_for(J.gd_ctas, J.rows_hint, 1), 512,
-                 direct ? (size_t)words * sizeof(uint32_t) : 0, next(), A, B, C, J, ctl, mask, (int)BIN_GD);
-    }
-    if (on(BIN_K8L)) launch_cluster_hash<SR, 14, 8>(A, B, C, J, ctl, mask, BIN_K8L, next(), num_sms);
-    if (on(BIN_K8)) launch_cluster_hash<SR, 13, 8>(A, B, C, J, ctl, mask, BIN_K8, next(), num_sms);
-    if (on(BIN_K4)) launch_cluster_hash<SR, 13, 4>(A, B, C, J, ctl, mask, BIN_K4, next(), num_sms);
-    if (on(BIN_K2)) launch_cluster_hash<SR, 13, 2>(A, B, C, J, ctl, mask, BIN_K2, next(), num_sms);
-    if (on(BIN_C16384)) launch_cta_hash<SR, 14>(A, B, C, J, ctl, mask, BIN_C16384, next(), num_sms);
-    if (on(BIN_C8192)) launch_cta_hash<SR, 13>(A, B, C, J, ctl, mask, BIN_C8192, next(), num_sms);
-    if (on(BIN_C4096)) launch_cta_hash<SR, 12>(A, B, C, J, ctl, mask, BIN_C4096, next(), num_sms);
-    if (on(BIN_C2048)) launch_cta_hash<SR, 11>(A, B, C, J, ctl, mask, BIN_C2048, next(), num_sms);
-    if (on(BIN_W1024)) launch_group_hash<SR, 10, 32, 4>(A, B, C, J, ctl, mask, BIN_W1024, next(), num_sms);
-    if (on(BIN_W512)) launch_group_hash<SR, 9, 32, 4>(A, B, C, J, ctl, mask, BIN_W512, next(), num_sms);
-    if (on(BIN_W256)) launch_group_hash<SR, 8, 32, 8>(A, B, C, J, ctl, mask, BIN_W256, next(), num_sms);
-    if (on(BIN_W128)) launch_group_hash<SR, 7, 32, 8>(A, B, C, J, ctl, mask, BIN_W128, next(), num_sms);
-    if (on(BIN_G16)) launch_group_hash<SR, 6, 16, 8>(A, B, C, J, ctl, mask, BIN_G16, next(), num_sms);
-    if (on(BIN_G8)) launch_group_hash<SR, 5, 8, 8>(A, B, C, J, ctl, mask, BIN_G8, next(), num_sms);
+        if (!on(bin)) return;
+        switch (bin) {
+            case BIN_G8: launch_group_hash<SR, 5, 8, 8>(A, B, C, J, ctl, mask, bin, next(), num_sms); break;
+            case BIN_G16: launch_group_hash<SR, 6, 16, 8>(A, B, C, J, ctl, mask, bin, next(), num_sms); break;
+            case BIN_W128: launch_group_hash<SR, 7, 32, 8>(A, B, C, J, ctl, mask, bin, next(), num_sms); break;
+            case BIN_W256: launch_group_hash<SR, 8, 32, 8>(A, B, C, J, ctl, mask, bin, next(), num_sms); break;
+            case BIN_W512: launch_group_hash<SR, 9, 32, 4>(A, B, C, J, ctl, mask, bin, next(), num_sms); break;
+            case BIN_W1024: launch_group_hash<SR, 10, 32, 4>(A, B, C, J, ctl, mask, bin, next(), num_sms); break;
+            case BIN_C2048: launch_cta_hash<SR, 11>(A, B, C, J, ctl, mask, bin, next(), num_sms); break;
+            case BIN_C4096: launch_cta_hash<SR, 12>(A, B, C, J, ctl, mask, bin, next(), num_sms); break;
+            case BIN_C8192: launch_cta_hash<SR, 13>(A, B, C, J, ctl, mask, bin, next(), num_sms); break;
+            case BIN_C16384: launch_cta_hash<SR, 14>(A, B, C, J, ctl, mask, bin, next(), num_sms); break;
+            case BIN_K2: launch_cluster_hash<SR, 13, 2>(A, B, C, J, ctl, mask, bin, next(), num_sms); break;
+            case BIN_K4: launch_cluster_hash<SR, 13, 4>(A, B, C, J, ctl, mask, bin, next(), num_sms); break;
+            case BIN_K8: launch_cluster_hash<SR, 13, 8>(A, B, C, J, ctl, mask, bin, next(), num_sms); break;
+            case BIN_K8L: launch_cluster_hash<SR, 14, 8>(A, B, C, J, ctl, mask, bin, next(), num_sms); break;
+        }
+    };
+    constexpr long long LONGEST_FIRST = 1LL << 17;  // columns of C
+    if (J.m >= LONGEST_FIRST)
+        for (int bin : {BIN_GD, BIN_K8L, BIN_K8, BIN_K4, BIN_K2, BIN_C16384, BIN_C8192, BIN_C4096, BIN_W1024, BIN_C2048,
+                        BIN_W512, BIN_W256, BIN_W128, BIN_G16, BIN_G8})
+            launch(bin);
+    else
+        for (int bin : {BIN_G16, BIN_G8, BIN_W128, BIN_W256, BIN_W512, BIN_W1024, BIN_C2048, BIN_C4096, BIN_C8192,
+                        BIN_C16384, BIN_K2, BIN_K4, BIN_K8, BIN_K8L, BIN_GD})
+            launch(bin);
     launch_s64();
 }
 
