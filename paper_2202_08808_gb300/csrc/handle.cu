@@ -1476,7 +1476,8 @@ void fill_rows_out(dspg_handle *h, DevMat &M, const MatView &V, int vs, const in
     };
     if (on_device) {
         if (rowptr != rp) CK(cudaMemcpyAsync(rowptr, rp, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToDevice, s));
-        rows_out(col, val);
+        DBuf<int32_t> c_l;
+        rows_out(col ? col : read_scratch(h->rd.c, c_l, nnz), val);  // no columns wanted: into scratch, as below
     } else {
         DBuf<int32_t> c_l;
         DBuf<char> v_l;
@@ -1625,10 +1626,12 @@ int64_t read_form(dspg_handle *h, const int32_t *rows_in, int64_t nr, int64_t *r
     DBuf<char> oval_l;
     int32_t *ocol = col;
     void *oval = val;
-    if (!on_device) {
+    if (!on_device || !col) {
         ocol_l.reserve(std::max<int64_t>(nnz, 1));
-        oval_l.reserve(std::max<int64_t>(nnz, 1) * h->vsize);
         ocol = ocol_l.p;
+    }
+    if (!on_device || !val) {
+        oval_l.reserve(std::max<int64_t>(nnz, 1) * h->vsize);
         oval = oval_l.p;
     }
     form_merge(h->sr, rows, n, prp.p, pcol.p, pval.p, xrp, h->xcol.p, h->xval.p, orp, ocol, oval, h->fs, s,

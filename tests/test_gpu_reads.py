@@ -254,3 +254,30 @@ def test_whole_read_while_an_asynchronous_batch_rewrites_rows(dspg):
         short = np.sum((np.diff(want[0]) > np.diff(orp)) & (np.diff(want[0]) <= 64))
         assert st["relocations"] > moved_a.sum() + short and st["compactions"] == 0
     g.close()
+
+
+@pytest.mark.parametrize("form", [False, True])
+@pytest.mark.parametrize("on_device", [0, 1])
+def test_reads_without_columns_or_without_values(dspg, form, on_device):
+    """col and val may be NULL in a fill call, in host and in device memory."""
+    import ctypes
+    import torch
+    sr = PLUS_TIMES_F64
+    rng = np.random.default_rng(8)
+    n = 90
+    A = _csr([rng.choice(n, size=int(rng.integers(0, 40)), replace=False) for _ in range(n)], n, sr, rng)
+    g = dspg.DynamicSpGEMM(A, **(dict(alpha=2.0, beta=1.0, X=A) if form else {}))
+    want = g.read_C()
+    lib = dspg.load()
+    dev = "cuda" if on_device else "cpu"
+    for with_col, with_val in ((True, False), (False, True), (False, False)):
+        rp = torch.zeros(n + 1, dtype=torch.int64, device=dev)
+        col = torch.full((want.col.size,), -7, dtype=torch.int32, device=dev)
+        val = torch.full((want.col.size,), -7.0, dtype=torch.float64, device=dev)
+        nnz = ctypes.c_int64()
+        assert lib.dspg_read_C(g._h, ctypes.byref(nnz), rp.data_ptr(), col.data_ptr() if with_col else None,
+                               val.data_ptr() if with_val else None, on_device, None) == 0
+        assert nnz.value == want.col.size and np.array_equal(rp.cpu().numpy(), want.rowptr)
+        assert np.array_equal(col.cpu().numpy(), want.col if with_col else np.full(want.col.size, -7))
+        assert np.array_equal(val.cpu().numpy(), want.val if with_val else np.full(want.col.size, -7.0))
+    g.close()
