@@ -295,7 +295,8 @@ int dspg_debug_build(void);
  * Buffers smaller than rows_cap < n or nnz_cap < nnz: DSPG_ERR_INVALID with
  * the sizes written (the caller grows and calls again).  Synchronises the
  * stream once when col and val are page-locked host memory, twice
- * otherwise.  Not for handles with alpha, beta or X (DSPG_ERR_STATE).
+ * otherwise (page-locked over all of nnz_cap entries, and aligned).  Not for
+ * handles with alpha, beta or X (DSPG_ERR_STATE).
  * Not part of the paper: the read a server makes after each batch. */
 dspg_status dspg_read_affected_C(dspg_handle *h, int64_t rows_cap, int64_t nnz_cap, int64_t *nrows_out,
                                  int64_t *nnz_out, int32_t *rows, int64_t *rowptr, int32_t *col, void *val,

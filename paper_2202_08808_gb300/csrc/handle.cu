@@ -1167,14 +1167,12 @@ void upload(dspg_handle *h, UpdWs &w, const dspg_updates *u, BatchIn &in, int k,
     // link, by the sort (its one reader), if its arrays are aligned for loads
     // and page-locked from their first byte to their last
     const void *dr = nullptr, *dc = nullptr, *dv = nullptr, *dp = nullptr;
-    const bool aligned = ((uintptr_t)ur | (uintptr_t)uc) % sizeof(int32_t) == 0 && (uintptr_t)u->val % h->vsize == 0;
-    if (!u->on_device && in.n <= kInPlace && aligned) {
-        const size_t n = (size_t)in.n;
-        auto view = [](const void *p, size_t bytes) { return range_view(device_view, const_cast<void *>(p), bytes); };
-        dr = view(ur, sizeof(int32_t) * n);
-        dc = dr ? view(uc, sizeof(int32_t) * n) : nullptr;
-        dv = dc ? view(u->val, (size_t)h->vsize * n) : nullptr;
-        dp = dv ? view(u->op, sizeof(uint8_t) * n) : nullptr;
+    if (!u->on_device && in.n <= kInPlace) {
+        auto view = [&](const void *p, size_t size) { return array_view(device_view, const_cast<void *>(p), in.n, size); };
+        dr = view(ur, sizeof(int32_t));
+        dc = dr ? view(uc, sizeof(int32_t)) : nullptr;
+        dv = dc ? view(u->val, h->vsize) : nullptr;
+        dp = dv ? view(u->op, sizeof(uint8_t)) : nullptr;
     }
     if (u->on_device) {
         in.row = ur;
@@ -2698,8 +2696,9 @@ dspg_status dspg_read_affected_C(dspg_handle *h, int64_t rows_cap, int64_t nnz_c
         // page-locked host buffers: the rows go straight into them, in column
         // order, with one synchronisation (unless R was not collected in
         // order, which the read finds on the device and leaves to the path below)
-        int32_t *dcol = rows && !on_device && h->direct_read && rows_cap >= n ? (int32_t *)device_view(col) : nullptr;
-        void *dval = (dcol && val && h->vsize) ? device_view(val) : nullptr;
+        int32_t *dcol = rows && !on_device && h->direct_read && rows_cap >= n
+                            ? (int32_t *)array_view(device_view, col, nnz_cap, sizeof(int32_t)) : nullptr;
+        void *dval = (dcol && val && h->vsize) ? array_view(device_view, val, nnz_cap, h->vsize) : nullptr;
         const bool direct = dcol && (!val || !h->vsize || dval);
         if (direct) w.res.reserve(1);
         // R in row order and its row pointers: two launches (each block scans
@@ -2707,8 +2706,8 @@ dspg_status dspg_read_affected_C(dspg_handle *h, int64_t rows_cap, int64_t nnz_c
         // rowptr as well on the direct path; with a larger chunk table, the
         // chunk scan, a gather of the lengths and their scan
         const bool two = nch <= read_nch_max();
-        int32_t *drows = direct && two ? (int32_t *)device_view(rows) : nullptr;
-        int64_t *drp = direct && two ? (int64_t *)device_view(rowptr) : nullptr;
+        int32_t *drows = direct && two ? (int32_t *)array_view(device_view, rows, n, sizeof(int32_t)) : nullptr;
+        int64_t *drp = direct && two ? (int64_t *)array_view(device_view, rowptr, n + 1, sizeof(int64_t)) : nullptr;
         if (two) {
             read_order_rowptr(h->wc.R.p, h->wc.rchunk.p, nch, n, nullptr, n, nullptr, h->C.len.p, w.r.p, lens,
                               w.chunk_cnt.p, w.chunk_ex.p + nch, rp, drows, drp, direct ? w.res.p : nullptr, s,
@@ -2798,10 +2797,10 @@ dspg_status dspg_apply_read_affected(dspg_handle *h, const dspg_updates *dA, con
     bool one = !h->bloom && h->direct_read && rows && rowptr && col && rows_cap >= 0 && nnz_cap >= 0 &&
                nch <= read_nch_max();
     if (one) {
-        drows = (int32_t *)device_view(rows);
-        drp = (int64_t *)device_view(rowptr);
-        dcol = (int32_t *)device_view(col);
-        dval = (val && h->vsize) ? device_view(val) : nullptr;
+        drows = (int32_t *)array_view(device_view, rows, rows_cap, sizeof(int32_t));
+        drp = drows ? (int64_t *)array_view(device_view, rowptr, rows_cap + 1, sizeof(int64_t)) : nullptr;
+        dcol = drp ? (int32_t *)array_view(device_view, col, nnz_cap, sizeof(int32_t)) : nullptr;
+        dval = (dcol && val && h->vsize) ? array_view(device_view, val, nnz_cap, h->vsize) : nullptr;
         one = drows && drp && dcol && (!val || !h->vsize || dval);
     }
     if (one) {

@@ -281,3 +281,36 @@ def test_reads_without_columns_or_without_values(dspg, form, on_device):
         assert np.array_equal(col.cpu().numpy(), want.col if with_col else np.full(want.col.size, -7))
         assert np.array_equal(val.cpu().numpy(), want.val if with_val else np.full(want.col.size, -7.0))
     g.close()
+
+
+@pytest.mark.parametrize("shift", [0, 2, 4])
+def test_affected_rows_into_arrays_off_their_alignment(dspg, shift):
+    """Page-locked result arrays that start `shift` bytes past an aligned
+    address get the same rows (through scratch where their values would be
+    misaligned), by both one-call reads."""
+    import torch
+    from workloads import random_batch
+    sr = PLUS_TIMES_F64
+    rng = np.random.default_rng(shift)
+    n = 500
+    A = _csr([rng.choice(n, size=int(rng.integers(0, 30)), replace=False) for _ in range(n)], n, sr, rng)
+    g = dspg.DynamicSpGEMM(A)
+    Ao = OMat.from_csr(A)
+
+    def pinned(count, dtype):
+        raw = torch.empty(count * np.dtype(dtype).itemsize + 64, dtype=torch.uint8, pin_memory=True).numpy()
+        return raw[shift: shift + count * np.dtype(dtype).itemsize].view(dtype)
+
+    out = (pinned(n, np.int32), pinned(n + 1, np.int64), pinned(n * n, np.int32), pinned(n * n, np.float64))
+    for t in range(3):
+        b = random_batch(n, n, 60, t, sr, A=Ao.to_csr())
+        _, got = g.apply_read_affected(b, out=out)
+        got = [x.copy() for x in got]
+        Ao.apply(b)
+        rows = g.last_affected()
+        want = Ao.multiply_rows(Ao, rows)
+        sabs = Ao.multiply_rows(Ao, rows, absval=True)[2]
+        for r in (got, g.read_affected(out=out)):
+            assert np.array_equal(r[0], rows)
+            assert_rows_match(*r[1:], *want, sabs, f"shift {shift}, batch {t}")
+    g.close()
