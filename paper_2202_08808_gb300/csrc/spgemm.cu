@@ -799,11 +799,11 @@ __device__ __forceinline__ int hash_acc(int32_t *keys, T *vals, int32_t j, T v) 
 // round meet each other, and what the claims cost is left.  Static products
 // of 30 million products, us with / without claims, for rows whose columns
 // are all different | as many as their products, at random | one block:
-//   group kernels, (+,.), 400 products a row     475 / 796 | 420 / 684 | 326 / 367
-//   group kernels, (min,+), 400                  427 / 433 | 377 / 375 | 260 / 252
-//   8192 slots, (+,.), 7744                      786 / 956 | 522 / 575 | 721 / 611
-//   16384 slots, (+,.), 14400                    789 / 945 | 605 / 656 | 1009 / 835
-//   16384 slots, (min,+), 14400                  771 / 823 | 551 / 565 | 373 / 389
+//   group kernels, (+,.), 400 products a row     491 / 752 | 416 / 617 | 333 / 329
+//   group kernels, (min,+), 400                  429 / 441 | 377 / 371 | 255 / 244
+//   8192 slots, (+,.), 7744                      785 / 966 | 525 / 584 | 720 / 605
+//   16384 slots, (+,.), 14400                    784 / 948 | 611 / 656 | 1005 / 831
+//   16384 slots, (min,+), 14400                  765 / 783 | 547 / 518 | 372 / 354
 // So the group kernels of (min,+), whose atomics are native, go without (300
 // edges of a squared R-MAT 18 in (min,+) 1907 to 1877 us); so do the 16384
 // slots of (+,.), which R-MAT batches do not notice (2416 us at scale 18).
