@@ -808,7 +808,8 @@ __device__ __forceinline__ int hash_acc(int32_t *keys, T *vals, int32_t j, T v) 
 // edges of a squared R-MAT 18 in (min,+) 1907 to 1877 us); so do the 16384
 // slots of (+,.), which R-MAT batches do not notice (2416 us at scale 18).
 // The 8192 slots keep them: exact sizing of R-MAT 17 is 1030 us with and 1150
-// without.
+// without.  The CTA tables of (min,+) keep them too: columns apart gain about
+// what shared ones lose, and batches of R-MAT 14 and 15 are 1 percent faster.
 template <int LOG_TS, typename T>
 __device__ __forceinline__ int hash_claim(int32_t *keys, T *vals, int32_t j, T v, int &fresh) {
     constexpr int TS = 1 << LOG_TS;
