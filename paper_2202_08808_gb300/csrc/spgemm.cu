@@ -347,27 +347,32 @@ __global__ void __launch_bounds__(256) k_size_bins(MatView A, MatView B, MatView
         }
         const bool lng = alen > SIZE_SHORT && !direct;
         long long ub = direct ? J.m : 0, bmax = 0;
-        if (valid && !lng && !direct)
+        if (valid && !lng && !direct) {
             // eight entries a step, all their loads in flight together; a row starts at a multiple of 4 entries, and
             // its room ends at one.  Past the row's end nothing is loaded: with the step's first entry looked up
             // again there, a million rows of 9 entries against 4096 rows of B took 286 us (102 with an entry at a
-            // time, 92 so), as all those lookups meet in the few L2 slices that hold B's lengths
-#pragma unroll 1
-            for (int a = 0; a < alen; a += 8) {
+            // time, 87 so), as all those lookups meet in the few L2 slices that hold B's lengths
+            auto step = [&](int a, auto whole) {
+                constexpr bool WHOLE = decltype(whole)::value;
                 const int4 k0 = __ldcg((const int4 *)(A.col + aoff + a));
-                const int4 k1 = a + 4 < alen ? __ldcg((const int4 *)(A.col + aoff + a + 4)) : k0;
+                const int4 k1 = WHOLE || a + 4 < alen ? __ldcg((const int4 *)(A.col + aoff + a + 4)) : k0;
                 const int32_t kk[8] = {k0.x, k0.y, k0.z, k0.w, k1.x, k1.y, k1.z, k1.w};
                 int32_t l[8];
 #pragma unroll
                 for (int u = 0; u < 8; u++)
-                    l[u] = a + u < alen && dcheck(ctl, kk[u] >= 0 && kk[u] < B.nrows, DBG_B_ROW, aoff + a + u)
+                    l[u] = (WHOLE || a + u < alen) && dcheck(ctl, kk[u] >= 0 && kk[u] < B.nrows, DBG_B_ROW, aoff + a + u)
                                ? __ldcg(B.len + kk[u]) : 0;
 #pragma unroll
                 for (int u = 0; u < 8; u++) {
                     ub += l[u];
                     bmax = l[u] > bmax ? l[u] : bmax;
                 }
-            }
+            };
+            int a = 0;
+#pragma unroll 1
+            for (; a + 8 <= alen; a += 8) step(a, std::true_type());
+            if (a < alen) step(a, std::false_type());
+        }
         if (valid && lng) {
             const int k = atomicAdd(&s_nmid, 1);
             s_mid[k] = (int)threadIdx.x;
