@@ -2351,10 +2351,10 @@ static void run_numeric_t(const MatView &A, const MatView &B, const MatView &C, 
     // it starts first; but while no row is long it only delays the kernels
     // that hold the bulk of the rows.  How long a row can get is what C's
     // width allows, so the line is drawn there.  Longest first / shortest
-    // first, us, squares of R-MAT graphs: scale 18, a batch of 600 entries 916 /
+    // first, us, squares of R-MAT graphs: scale 18, a batch of 600 entries 926 /
     // 965; scale 17, 250 edges and the read 1798 / 1828 in (+,.), 1176 / 1177 in
     // (min,+); scale 16, 100 edges and the read 712 / 699; scale 15, a batch of
-    // 1000 entries 287 / 280, scale 14 of one entry 114 / 103.  The global dense
+    // 1000 entries 301 / 280, scale 14 of one entry 108 / 103.  The global dense
     // bin is always launched: rows of bins that are off go there.
     auto launch = [&](int bin) {
         if (bin == BIN_GD) {
@@ -2389,7 +2389,7 @@ static void run_numeric_t(const MatView &A, const MatView &B, const MatView &C, 
     };
     constexpr long long LONGEST_FIRST = 1LL << 17;  // columns of C
     if (J.m >= LONGEST_FIRST)
-        for (int bin : {BIN_GD, BIN_K8L, BIN_K8, BIN_K4, BIN_K2, BIN_C16384, BIN_C8192, BIN_C4096, BIN_W1024, BIN_C2048,
+        for (int bin : {BIN_GD, BIN_K8L, BIN_K8, BIN_K4, BIN_K2, BIN_C16384, BIN_C8192, BIN_C4096, BIN_C2048, BIN_W1024,
                         BIN_W512, BIN_W256, BIN_W128, BIN_G16, BIN_G8})
             launch(bin);
     else
